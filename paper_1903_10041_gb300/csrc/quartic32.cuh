@@ -238,6 +238,159 @@ __device__ __forceinline__ double quartic_min64_seeded(double A, double B, doubl
 }
 
 // ---------------------------------------------------------------------------
+// Step (a) of one element in FP64, in the factored form of its terms of L:
+//   (a_2/q + rho_3/2) x^2 + (a_1/q - rho_3 phi) x + (rho_1/2) (b_2 x^2 + b_1 x - u)^2
+// (plus the rho_4 terms at k = 0).  Half its derivative is
+//   H(x) = C x + Dh + hr1 e g',  e = b_2 x^2 + b_1 x - u,  g' = 2 b_2 x + b_1,  hr1 = rho_1/2,
+// six FP64 instructions, against twelve to expand A, B, C, D and three per
+// Horner evaluation.  The root is found in FP32 (closed form of the cubic in
+// z = x + b_1/(2 b_2), where it is already depressed, then a Newton step on H)
+// and refined by two FP64 Newton steps with one FP32 slope: each multiplies
+// the error by the slope's relative error.  21 FP64-pipe instructions per
+// element with losses and 7 without, where expanding the quartic and
+// converting and comparing on the FP64 pipe took about 80 and 25.
+// ---------------------------------------------------------------------------
+struct Elem64 {
+    double b2, b1, u, C, Dh, hr1;
+};
+
+// The FP64 closed form of Algorithm 1, out of line: the trig and triple-root
+// branches, a discriminant FP32 cannot certify, values outside the FP32 range, a
+// Newton step that did not settle.
+static __device__ __noinline__ double elem_min64(Elem64 p, double lo, double hi, int paper_mode)
+{
+    const double A = p.hr1 * p.b2 * p.b2, B = 2.0 * p.hr1 * p.b2 * p.b1;
+    const double C = p.C + p.hr1 * (p.b1 * p.b1 - 2.0 * p.b2 * p.u), D = 2.0 * (p.Dh - p.hr1 * p.b1 * p.u);
+    return quartic_min64(A, B, C, D, lo, hi, paper_mode);
+}
+
+// One Newton step on H in FP32, then 1 / H' at the new point; false where H'
+// is not positive there or a value left the FP32 range.
+__device__ __forceinline__ bool elem_polish32(float b2, float b1, float u, float C, float Dh, float hr1, float y,
+                                              float &x, float &r)
+{
+    const float t = fmaf(b2, y, b1), e = fmaf(t, y, -u), gp = fmaf(b2, y, t);
+    const float dx = fmaf(e * gp, hr1, fmaf(C, y, Dh)) * rcp_fast(fmaf(hr1, fmaf(gp, gp, 2.0f * b2 * e), C));
+    if (fabsf(dx) <= 0.0625f * (fabsf(y) + 1.0f)) y -= dx;
+    const float t1 = fmaf(b2, y, b1), e1 = fmaf(t1, y, -u), gp1 = fmaf(b2, y, t1);
+    const float s = fmaf(hr1, fmaf(gp1, gp1, 2.0f * b2 * e1), C);
+    x = y;
+    r = rcp_fast(s);
+    return s > 0.0f && isfinite(x) && isfinite(r) && r >= 1.2e-38f;
+}
+
+// The minimiser's FP32 root where H has three real roots (Delta < 0
+// certified, Q < 0): with z = x + b_1/(2 b_2) the quartic is z^4/4 + (3/2) Q z^2
+// - 2 R z up to scale, so
+//  * where [lo, hi] lies right of z = sqrt(-Q) (left of -sqrt(-Q)), H
+//    increases on it and the constrained minimiser is the clamped largest
+//    (smallest) root;
+//  * the lower of the two minima is the one on the side of R's sign; it is
+//    the constrained minimiser too if it lies inside (lo, hi).
+// Anything else (a minimum outside the interval that holds the other) is left
+// to the FP64 closed form.  dR bounds R's error.  Out of line: rare.
+static __device__ __noinline__ bool elem_trig32(float Q, float R, float dR, float b3, float lo, float hi,
+                                                int paper_mode, float &y)
+{
+    const float nQ = -Q, s = sqrt_fast(nQ);
+    const float mlo = 1.0e-5f * (fabsf(lo) + fabsf(b3) + 1.0f), mhi = 1.0e-5f * (fabsf(hi) + fabsf(b3) + 1.0f);
+    int side = 0;
+    if (!paper_mode) {
+        if (lo + b3 - mlo > 1.0001f * s) side = 1;
+        else if (hi + b3 + mhi < -1.0001f * s) side = -1;
+    }
+    const bool basin = side != 0;
+    if (!basin) {
+        if (!(fabsf(R) > dR)) return false;
+        side = R > 0.0f ? 1 : -1;
+    }
+    const float Rs = side > 0 ? R : -R;
+    const float arg = fminf(fmaxf(Rs * rsqrtf(nQ * nQ * nQ), -1.0f), 1.0f);
+    const float z = 2.0f * s * __cosf(acosf(arg) * (1.0f / 3.0f));
+    y = (side > 0 ? z : -z) - b3;
+    return basin || paper_mode || (y > lo + mlo && y < hi - mhi);
+}
+
+// FP32 root of H (x) and 1 / H'(x) (r) that the minimiser is refined from:
+// the quadratic case (b_2 = 0), the Cardano branch with Delta > 0 certified,
+// and the trig branch with Delta < 0 certified where elem_trig32 can tell the root.
+// Q and R carry the rounding of b_2, b_1, u, C, Dh to FP32, that of their own
+// operations and two reciprocals off by 2 ulp: |dQ| <= 24 v mQ, |dR| <= 17 v mR
+// (v = 2^-24, mQ, mR the sums of the terms' magnitudes), so |dDelta| <=
+// v (76 Q^2 mQ + 37 |R| mR); the bound takes 128 v for both.
+__device__ __forceinline__ bool elem_seed32(float b2, float b1, float u, float C, float Dh, float hr1, float lo,
+                                            float hi, int paper_mode, float &x, float &r)
+{
+    const float hb1 = hr1 * b1;
+    if (b2 == 0.0f) {
+        r = rcp_fast(fmaf(hb1, b1, C));
+        x = fmaf(hb1, u, -Dh) * r;
+        return isfinite(x) && r >= 1.2e-38f;
+    }
+    const float b3 = 0.5f * b1 * rcp_fast(b2);
+    const float v = 0.5f * b1 * b3;                 // b_1^2 / (4 b_2)
+    const float k2 = (hr1 + hr1) * b2;
+    const float inv = rcp_fast(k2 * b2), inv3 = inv * (1.0f / 3.0f), inv2 = 0.5f * inv;
+    const float Q = (C - k2 * (u + v)) * inv3, R = (C * b3 - Dh) * inv2;
+    const float mQ = (C + k2 * (fabsf(u) + fabsf(v))) * inv3, mR = (C * fabsf(b3) + fabsf(Dh)) * inv2;
+    const float Qs = Q * Q;
+    const float Dl = fmaf(Qs, Q, R * R);
+    const float bound = 7.68e-6f * fmaf(Qs, mQ, fabsf(R) * mR);
+    float y;
+    if (Dl > bound) {
+        const float sq = sqrt_fast(Dl);
+        const float S = cbrt_fast(R >= 0.0f ? R + sq : R - sq);
+        y = S - Q * rcp_fast(S) - b3;
+    } else if (!(Dl < -bound) || !elem_trig32(Q, R, 2.0e-6f * mR, b3, lo, hi, paper_mode, y)) {
+        return false;
+    }
+    return elem_polish32(b2, b1, u, C, Dh, hr1, y, x, r);
+}
+
+// The settled test of two Newton steps d0, d1 of a refined root: the second
+// step's own error is d1 times the ratio of the steps.
+__device__ __forceinline__ bool newton_settled(float d0, float d1, float x)
+{
+    const float s = fabsf(x) + 1.0f, a = fabsf(d1);
+    return a <= 1.0e-12f * s || (a <= 1.0e-10f * s && a <= 1.0e-5f * fabsf(d0));
+}
+
+// The constrained minimiser of an element with losses (b_2 or b_1 not zero).
+__device__ __forceinline__ double elem_min64_seeded(const Elem64 &p, float hr1f, double lo, double hi, int paper_mode)
+{
+    float xf, rf;
+    if (elem_seed32(f64_to_f32_int(p.b2), f64_to_f32_int(p.b1), f64_to_f32_int(p.u), f64_to_f32_int(p.C),
+                    f64_to_f32_int(p.Dh), hr1f, f64_to_f32_int(lo), f64_to_f32_int(hi), paper_mode, xf, rf)) {
+        const double r = f32_to_f64_int(rf);
+        double x = f32_to_f64_int(xf);
+        float d[2];
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const double w = fma(p.b2, x, p.b1), e = fma(w, x, -p.u), gp = fma(p.b2, x, w);
+            const double H = fma(e * gp, p.hr1, fma(p.C, x, p.Dh));
+            x = fma(-H, r, x);
+            d[t] = f64_to_f32_int(H) * rf;
+        }
+        if (newton_settled(d[0], d[1], xf)) return clamp_ord(x, lo, hi);
+    }
+    return elem_min64(p, lo, hi, paper_mode);
+}
+
+// The same without losses: H(x) = C x + Dh.
+__device__ __forceinline__ double elem_min64_linear(double C, double Dh, double lo, double hi)
+{
+    const float Cf = f64_to_f32_int(C), rf = rcp_fast(Cf), xf = -f64_to_f32_int(Dh) * rf;
+    if (rf >= 1.2e-38f && isfinite(rf) && isfinite(xf)) {
+        const double r = f32_to_f64_int(rf);
+        double x = f32_to_f64_int(xf);
+        x = fma(-fma(C, x, Dh), r, x);
+        x = fma(-fma(C, x, Dh), r, x);
+        return clamp_ord(x, lo, hi);
+    }
+    return clampd(-Dh / C, lo, hi);
+}
+
+// ---------------------------------------------------------------------------
 // Packed pair variant: the two columns of a vector in one float2, on the
 // paired FP32 instructions (FADD2 / FMUL2 / FFMA2: two lanes per issue, the
 // same rounding per lane as the scalar operations).  The common cases run

@@ -38,6 +38,43 @@ __device__ __forceinline__ float rcp_approx_f32(float v)
     return r;
 }
 
+// On this GPU every instruction of the FP64 pipe (fused multiply-adds, but
+// also comparisons and conversions from or to FP32) holds a scheduler's FP64
+// unit for 64 cycles (measured; an FP32 or integer instruction 1-2), so the
+// FP64 element update does its comparisons and conversions on the integer
+// pipes.
+
+// (float)v, rounded to nearest (halves away from zero); magnitudes below the
+// FP32 normal range give a signed zero, above it (and infinities, NaN) an infinity.
+__device__ __forceinline__ float f64_to_f32_int(double v)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v) + 0x10000000ull;
+    const unsigned hi = (unsigned)(b >> 32), ah = hi & 0x7fffffffu;
+    const unsigned f = ((unsigned)(b >> 29) - (896u << 23)) & 0x7fffffffu;
+    const unsigned r = ah < (897u << 20) ? 0u : (ah >= (1151u << 20) ? 0x7f800000u : f);
+    return __uint_as_float(r | (hi & 0x80000000u));
+}
+// (double)v, exact, for a zero or a normal v (a denormal gives a signed zero).
+__device__ __forceinline__ double f32_to_f64_int(float v)
+{
+    const unsigned b = __float_as_uint(v), a = b & 0x7fffffffu;
+    const bool z = a < 0x00800000u;
+    return __hiloint2double((int)((b & 0x80000000u) | (z ? 0u : (a >> 3) + (896u << 20))), (int)(z ? 0u : b << 29));
+}
+// Doubles as integers in the order of their values (no NaN; -0 before +0).
+__device__ __forceinline__ long long ord64(double v)
+{
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double clamp_ord(double v, double lo, double hi)
+{
+    const long long k = ord64(v);
+    return k < ord64(lo) ? lo : (k > ord64(hi) ? hi : v);
+}
+__device__ __forceinline__ double max_ord(double a, double b) { return ord64(a) < ord64(b) ? b : a; }
+__device__ __forceinline__ double min_ord(double a, double b) { return ord64(b) < ord64(a) ? b : a; }
+
 // 1/a: FP32 seed (relative error below 2^-22), then two Newton steps
 // r <- r + r (1 - a r), each squaring the relative error.  Operands outside
 // the FP32 normal range take the FP64 division.
