@@ -54,8 +54,12 @@ struct Sm {
     double *x1n;  // [kMaxM]
     double *red;  // [kSingleWarpsMax][kMaxM][3]
     double *mx;   // [kSingleWarpsMax][8]
-    double *bc;   // [16] broadcast
+    double *bc;   // [16] broadcast: [0] r, [1] sigma, [2] adaptation factor, [3] kappa, [4..6] rho_3/2, rho_4/2,
+                  //      rho_1/2, [7] int flags of a check (converged, penalties changed), [8..9] floats rho_1,
+                  //      rho_3, rho_4, rho_1/2
     int *segof;   // [kSingleWarpsMax] segment (within the pass) of each warp
+    int *rfirst;  // [q] first CTA whose columns touch row j
+    int *rcnt;    // [q] how many do
     float *uoff;  // [mq] zeta + lambda in FP32 (mixed variants)
     float *x1nu;  // [mq] x1 + nu in FP32 (mixed variants)
     double *zl;   // [mq] zeta + lambda (FP64 variant; the storage of uoff, x1nu)
@@ -68,7 +72,7 @@ __host__ __device__ inline size_t single_carve_bytes(int m, int q)
     const int mq = m * q;
     const size_t b = sizeof(double) * ((size_t)scal_size(m, q) + mq + kMaxM + kSingleWarpsMax * kMaxM * 3 +
                                        kSingleWarpsMax * 8 + 16 + kSingleWarpsMax) +
-                     sizeof(float) * 2 * (size_t)mq;
+                     sizeof(float) * 2 * (size_t)mq + sizeof(int) * 2 * (size_t)q;
     return (b + 15) / 16 * 16;
 }
 
@@ -100,28 +104,39 @@ __device__ __forceinline__ Sm carve(double *base, int m, int q)
     s.uoff = (float *)t;
     s.x1nu = s.uoff + mq;
     s.zl = t;
+    s.rfirst = (int *)(t + mq);
+    s.rcnt = s.rfirst + q;
     return s;
 }
 
-// Block-wide max of up to 8 non-negative values; every thread gets the results in v[].
-template <int NV, int NWP> __device__ __forceinline__ void block_max(double *v, const Sm &sm)
+// Warp sums (or maxima, minima) of M values per lane at once: while more than
+// one value is left, a step halves the values by keeping one half in the
+// lanes with the step's bit clear and the other in those with it set, so M
+// values take M - 1 + log2(32 / M) combinations instead of 5 M.  The total of
+// value slot_of<M>(lane) ends up in every lane of its group of 32 / M.
+template <int M> __device__ __forceinline__ int slot_of(int lane)
 {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    return M == 2 ? lane >> 4 : (M == 4 ? lane >> 3 : lane >> 2);
+}
+template <int M, class T, class F> __device__ __forceinline__ T warp_many(T *v, F comb)
+{
+    const int lane = threadIdx.x & 31;
+    int o = 16;
 #pragma unroll
-    for (int t = 0; t < NV; ++t) {
-        double r = warp_max_nonneg(v[t]);
-        if (lane == 0) sm.mx[w * 8 + t] = r;
-    }
-    __syncthreads();
-    if (threadIdx.x < NV) {
-        double r = 0.0;
-        for (int ww = 0; ww < NWP; ++ww) r = max_nonneg(r, sm.mx[ww * 8 + threadIdx.x]);
-        sm.bc[threadIdx.x] = r;
-    }
-    __syncthreads();
+    for (int c = M; c > 1; c >>= 1) {
+        const bool up = (lane & o) != 0;
 #pragma unroll
-    for (int t = 0; t < NV; ++t) v[t] = sm.bc[t];
-    __syncthreads();
+        for (int t = 0; t < M / 2; ++t)
+            if (t < c / 2) {
+                const T keep = up ? v[t + c / 2] : v[t], send = up ? v[t] : v[t + c / 2];
+                v[t] = comb(keep, send, o);
+            }
+        o >>= 1;
+    }
+    T r = v[0];
+#pragma unroll
+    for (int u = 16 / M; u > 0; u >>= 1) r = comb(r, r, u);
+    return r;
 }
 
 // Per-iteration constants of the FP64 element update, the same in every thread.
@@ -160,7 +175,7 @@ __device__ __forceinline__ void column64(const SingleArgs &a, const Sm &sm, cons
     const size_t col = (size_t)j * ld + k;
     const double st = Sv[col], yv = Y[col];
     double mu = MU[col];
-    if (mu_div != 1.0) mu = mu / mu_div;
+    if (__double_as_longlong(mu_div) != 0x3ff0000000000000ll) mu = mu / mu_div; // not 1.0
 #pragma unroll
     for (int i = M - 2; i >= 0; --i)
         if (i + 1 < m) suf[i] = i + 2 < m ? xt[i + 1] + suf[i + 1] : xt[i + 1];
@@ -235,7 +250,7 @@ struct SegPlan {
     int j;          // row of this warp's segment
     int seg;        // its index within the pass (j - jb)
     int lw, nw;     // this warp's index among the segment's warps, their count
-    int64_t s0, s1; // the segment's columns [s0, s1)
+    int kb, ke;     // the segment's columns k of row j
 };
 
 template <int NWP>
@@ -265,8 +280,9 @@ __device__ __forceinline__ SegPlan seg_plan(int64_t c0, int64_t c1, int64_t rs, 
         p.nw = whi - wlo;
         p.j = jb + p.seg;
     }
-    p.s0 = max(c0, (int64_t)p.j * rs);
-    p.s1 = min(c1, (int64_t)(p.j + 1) * rs);
+    const int64_t r0 = (int64_t)p.j * rs;
+    p.kb = (int)(max(c0, r0) - r0);
+    p.ke = (int)(min(c1, r0 + rs) - r0);
     return p;
 }
 
@@ -284,7 +300,7 @@ __device__ __noinline__ int pass_rows(int64_t c0, int64_t c1, int64_t rs, int jf
     for (int w = 0; w < NWP; ++w) {
         const SegPlan sp = seg_plan<NWP>(c0, c1, rs, jf, jl, w);
         if (sp.lw != 0) continue;
-        const int64_t v = (sp.s1 - sp.s0 + unit - 1) / unit;
+        const int64_t v = (sp.ke - sp.kb + unit - 1) / unit;
         conc = max(conc, (v + 32 * sp.nw - 1) / (32 * sp.nw));
         seq4 += 4 * ((v + 32 * NWP - 1) / (32 * NWP));
     }
@@ -304,119 +320,167 @@ __device__ __forceinline__ void cta_columns(const SingleArgs &a, int unit, int64
     }
 }
 
-// CTAs whose columns touch row j.
-__device__ __forceinline__ int row_ctas(const SingleArgs &a, int j)
+// CTAs whose columns touch row j: the first and how many.
+__device__ __forceinline__ void row_ctas(const SingleArgs &a, int j, int &first, int &cnt)
 {
-    if (a.pieces > 0) return a.pieces;
+    if (a.pieces > 0) {
+        first = j * a.pieces;
+        cnt = a.pieces;
+        return;
+    }
     const int64_t rbeg = (int64_t)j * a.rs;
-    return (int)((rbeg + a.rs - 1) / a.chunk - rbeg / a.chunk) + 1;
+    first = (int)(rbeg / a.chunk);
+    cnt = (int)((rbeg + a.rs - 1) / a.chunk) - first + 1;
 }
 
 // Partial record of row j written by this CTA (position among the CTAs
 // touching row j, in column order).
-__device__ __forceinline__ double *seg_record(const SingleArgs &a, int par, int j)
+__device__ __forceinline__ double *seg_record(const SingleArgs &a, const Sm &sm, int par, int j)
 {
-    const int pos = a.pieces > 0 ? (int)blockIdx.x % a.pieces
-                                 : (int)blockIdx.x - (int)(((int64_t)j * a.rs) / a.chunk);
-    return a.part + ((size_t)(par * a.q + j) * a.nbmax + pos) * a.m * 4;
+    return a.part + ((size_t)(par * a.q + j) * a.nbmax + ((int)blockIdx.x - sm.rfirst[j])) * a.m * 4;
 }
 
-// Reduction of one pass of row segments into their partial records: warp
-// sums by shuffles, then per (segment, source) the sum over that segment's
-// warps in warp order.
+// Reduction of one pass of row segments into their partial records, and (on
+// check iterations) of the CTA's column maxima: warp sums of all sources at
+// once by shuffles, then per (segment, source) the sum over that segment's
+// warps by the 16 lanes of a half warp, in a fixed order.
 template <int M, int NWP>
-__device__ __forceinline__ void flush_segments(const SingleArgs &a, int par, int jb, const double *gs,
-                                               const double *dmx, const double *dmn, bool check, int m,
+__device__ __forceinline__ void flush_segments(const SingleArgs &a, int par, int jb, int ns, double *gs, double *dmx,
+                                               double *dmn, double cm_r, double cm_s, bool check, int m,
                                                const SegPlan &sp, const Sm &sm)
 {
+    static_assert(NWP <= 16, "a half warp covers the warps");
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < M; ++i)
-        if (i < m) {
-            double v = warp_sum(gs[i]);
-            double hi = check ? warp_max(dmx[i]) : 0.0;
-            double lo = check ? warp_min(dmn[i]) : 0.0;
-            if (lane == 0) {
-                sm.red[(w * kMaxM + i) * 3 + 0] = v;
-                sm.red[(w * kMaxM + i) * 3 + 1] = hi;
-                sm.red[(w * kMaxM + i) * 3 + 2] = lo;
-            }
+    auto add = [](double k, double s, int o) { return k + __shfl_xor_sync(0xffffffffu, s, o); };
+    auto mx = [](double k, double s, int o) { return max_ord(k, __shfl_xor_sync(0xffffffffu, s, o)); };
+    auto mn = [](double k, double s, int o) { return min_ord(k, __shfl_xor_sync(0xffffffffu, s, o)); };
+    const int src = slot_of<M>(lane);
+    const double v = warp_many<M>(gs, add);
+    if (lane % (32 / M) == 0) sm.red[(w * kMaxM + src) * 3] = v;
+    if (check) {
+        const double hi = warp_many<M>(dmx, mx), lo = warp_many<M>(dmn, mn);
+        cm_r = warp_max_nonneg(cm_r);
+        cm_s = warp_max_nonneg(cm_s);
+        if (lane % (32 / M) == 0) {
+            sm.red[(w * kMaxM + src) * 3 + 1] = hi;
+            sm.red[(w * kMaxM + src) * 3 + 2] = lo;
         }
-    if (lane == 0) sm.segof[w] = sp.seg;
-    __syncthreads();
-    if (threadIdx.x < NWP * m) {
-        const int sg = threadIdx.x / m, i = threadIdx.x - sg * m;
-        double v = 0.0, hi = -INFINITY, lo = INFINITY;
-        bool any = false;
-        for (int ww = 0; ww < NWP; ++ww)
-            if (sm.segof[ww] == sg) {
-                any = true;
-                v += sm.red[(ww * kMaxM + i) * 3 + 0];
-                hi = fmax(hi, sm.red[(ww * kMaxM + i) * 3 + 1]);
-                lo = fmin(lo, sm.red[(ww * kMaxM + i) * 3 + 2]);
-            }
-        if (any) {
-            double *rec = seg_record(a, par, jb + sg);
-            rec[i * 4 + 0] = v;
-            rec[i * 4 + 1] = hi;
-            rec[i * 4 + 2] = lo;
+        if (lane == 0) {
+            sm.mx[w * 8] = cm_r;
+            sm.mx[w * 8 + 1] = cm_s;
         }
     }
+    if (lane == 0) sm.segof[w] = sp.seg;
     __syncthreads();
+    const int hl = lane & 15;
+    for (int t = 2 * w + (lane >> 4); t - (lane >> 4) < ns * m; t += 2 * NWP) { // a half warp per (segment, source)
+        const int sg = t / m, i = t - sg * m;
+        const bool in = t < ns * m && hl < NWP && sm.segof[hl < NWP ? hl : 0] == sg;
+        double r = in ? sm.red[(hl * kMaxM + i) * 3] : 0.0;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+        double hi = 0.0, lo = 0.0;
+        if (check) {
+            hi = in ? sm.red[(hl * kMaxM + i) * 3 + 1] : -INFINITY;
+            lo = in ? sm.red[(hl * kMaxM + i) * 3 + 2] : INFINITY;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) {
+                hi = mx(hi, hi, o);
+                lo = mn(lo, lo, o);
+            }
+        }
+        if (hl == 0 && t < ns * m) {
+            double *rec = seg_record(a, sm, par, jb + sg);
+            rec[i * 4 + 0] = r;
+            if (check) {
+                rec[i * 4 + 1] = hi;
+                rec[i * 4 + 2] = lo;
+            }
+        }
+    }
 }
 
 // Mixed variant, on the FP32 pipes: float-float sums and FP32 max / min in
 // a fixed order; only the finished records are converted to FP64.
 template <int M, int NWP>
-__device__ __forceinline__ void flush_segments32(const SingleArgs &a, int par, int jb, const float2 *ghi,
-                                                 const float2 *glo, const float *fmx, const float *fmn, bool check,
-                                                 int m, const SegPlan &sp, const Sm &sm)
+__device__ __forceinline__ void flush_segments32(const SingleArgs &a, int par, int jb, int ns, const float2 *ghi,
+                                                 const float2 *glo, float *fmx, float *fmn, float cm_r, float cm_s,
+                                                 bool check, int m, const SegPlan &sp, const Sm &sm)
 {
     float *red = (float *)sm.red; // [NWP][kMaxM][4] floats
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    auto add = [](FF k, FF s, int o) {
+        return ff_add(k, FF{__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o)});
+    };
+    auto mx = [](float k, float s, int o) { return fmaxf(k, __shfl_xor_sync(0xffffffffu, s, o)); };
+    auto mn = [](float k, float s, int o) { return fminf(k, __shfl_xor_sync(0xffffffffu, s, o)); };
+    FF g[M];
 #pragma unroll
-    for (int i = 0; i < M; ++i)
-        if (i < m) {
-            FF v = lanes_sum(ghi[i], glo[i]);
-            float hi = fmx[i], lo = fmn[i];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const FF u = {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
-                v = ff_add(v, u);
-                if (check) {
-                    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-                    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-                }
-            }
-            if (lane == 0) {
-                red[(w * kMaxM + i) * 4 + 0] = v.hi;
-                red[(w * kMaxM + i) * 4 + 1] = v.lo;
-                red[(w * kMaxM + i) * 4 + 2] = hi;
-                red[(w * kMaxM + i) * 4 + 3] = lo;
-            }
+    for (int i = 0; i < M; ++i) g[i] = lanes_sum(ghi[i], glo[i]);
+    const int src = slot_of<M>(lane);
+    const FF v = warp_many<M>(g, add);
+    float *rw = red + (w * kMaxM + src) * 4;
+    if (lane % (32 / M) == 0) {
+        rw[0] = v.hi;
+        rw[1] = v.lo;
+    }
+    if (check) {
+        const float hi = warp_many<M>(fmx, mx), lo = warp_many<M>(fmn, mn);
+        cm_r = warp_max(cm_r);
+        cm_s = warp_max(cm_s);
+        if (lane % (32 / M) == 0) {
+            rw[2] = hi;
+            rw[3] = lo;
         }
-    if (lane == 0) sm.segof[w] = sp.seg;
-    __syncthreads();
-    if (threadIdx.x < NWP * m) {
-        const int sg = threadIdx.x / m, i = threadIdx.x - sg * m;
-        FF v = {0.0f, 0.0f};
-        float hi = -INFINITY, lo = INFINITY;
-        bool any = false;
-        for (int ww = 0; ww < NWP; ++ww)
-            if (sm.segof[ww] == sg) {
-                any = true;
-                v = ff_add(v, FF{red[(ww * kMaxM + i) * 4 + 0], red[(ww * kMaxM + i) * 4 + 1]});
-                hi = fmaxf(hi, red[(ww * kMaxM + i) * 4 + 2]);
-                lo = fminf(lo, red[(ww * kMaxM + i) * 4 + 3]);
-            }
-        if (any) {
-            double *rec = seg_record(a, par, jb + sg);
-            rec[i * 4 + 0] = (double)v.hi + (double)v.lo;
-            rec[i * 4 + 1] = check ? (double)hi : 0.0;
-            rec[i * 4 + 2] = check ? (double)lo : 0.0;
+        if (lane == 0) {
+            sm.mx[w * 8] = f32_to_f64_int(cm_r);
+            sm.mx[w * 8 + 1] = f32_to_f64_int(cm_s);
         }
     }
+    if (lane == 0) sm.segof[w] = sp.seg;
     __syncthreads();
+    const int hl = lane & 15;
+    for (int t = 2 * w + (lane >> 4); t - (lane >> 4) < ns * m; t += 2 * NWP) { // a half warp per (segment, source)
+        const int sg = t / m, i = t - sg * m;
+        const bool in = t < ns * m && hl < NWP && sm.segof[hl < NWP ? hl : 0] == sg;
+        const float *rr = red + (hl * kMaxM + i) * 4;
+        FF r = in ? FF{rr[0], rr[1]} : FF{0.0f, 0.0f};
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) r = add(r, r, o);
+        float hi = 0.0f, lo = 0.0f;
+        if (check) {
+            hi = in ? rr[2] : -INFINITY;
+            lo = in ? rr[3] : INFINITY;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) {
+                hi = mx(hi, hi, o);
+                lo = mn(lo, lo, o);
+            }
+        }
+        if (hl == 0 && t < ns * m) {
+            double *rec = seg_record(a, sm, par, jb + sg);
+            rec[i * 4 + 0] = f32_to_f64_int(r.hi) + f32_to_f64_int(r.lo);
+            if (check) {
+                rec[i * 4 + 1] = f32_to_f64_int(hi);
+                rec[i * 4 + 2] = f32_to_f64_int(lo);
+            }
+        }
+    }
+}
+
+// The values derived from the penalties that the next iterations read (by one thread).
+__device__ __forceinline__ void derive_penalties(const Sm &sm, int n)
+{
+    const double r1 = sm.rho[0], r2 = sm.rho[1], r3 = sm.rho[2], r4 = sm.rho[3];
+    sm.bc[3] = r2 / (r1 + (double)n * r2); // kappa of step (b)
+    sm.bc[4] = 0.5 * r3;
+    sm.bc[5] = 0.5 * r4;
+    sm.bc[6] = 0.5 * r1;
+    float *f = (float *)(sm.bc + 8);
+    f[0] = (float)r1;
+    f[1] = (float)r3;
+    f[2] = (float)r4;
+    f[3] = (float)(0.5 * r1);
 }
 
 // MINB: CTAs per SM the register budget is sized for.  FP64 takes 1 (its
@@ -441,34 +505,43 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
             sm.zl[pr] = sm.zeta[pr] + sm.lam[pr];
         }
     }
+    for (int j = threadIdx.x; j < q; j += NT) row_ctas(a, j, sm.rfirst[j], sm.rcnt[j]);
+    if (threadIdx.x == 0) derive_penalties(sm, n);
+    const double iq64 = 1.0 / (double)q, nd = (double)n;
+    const float iq = 1.0f / (float)q;
+    // lanes that share the records of one pair in the scalar phase
+    int gsh = 0;
+    while ((2 << gsh) <= a.nbmax && gsh < 5 && (mq << (gsh + 1)) <= NT) ++gsh;
+    const int G = 1 << gsh;
+    bool cold = sm.flags[0] != 0.0;
+    double mu_div = sm.flags[1];
     __syncthreads();
-    const double iq64 = 1.0 / (double)q;
 
     int64_t c0, c1;
     cta_columns(a, MIXED ? VW : 1, c0, c1);
     const int jf = (int)(c0 / rs), jl = (int)((c1 - 1) / rs);
     const int prows = pass_rows<NWP>(c0, c1, rs, jf, jl, MIXED ? VW : 1);
+    const SegPlan sp0 = seg_plan<NWP>(c0, c1, rs, jf, min(jl, jf + prows - 1), threadIdx.x >> 5);
     unsigned nbar = 0;
     unsigned esc = 0;
     bool ok = true, conv = false;
-    int it;
+    int it, ncheck = a.check_every; // iterations up to the next check
     double res[7] = {0, 0, 0, 0, 0, 0, 0}; // r1 r2 r3 r4 s1 s2 s3 (unscaled s)
     double r_last = INFINITY, s_last = INFINITY;
-    double kappa = sm.rho[1] / (sm.rho[0] + (double)n * sm.rho[1]); // step (b); renewed when rho changes
+    const float *fp = (const float *)(sm.bc + 8);
 
     for (it = 1; it <= a.max_iter; ++it) {
-        const bool check = (it % a.check_every == 0) || (it == a.max_iter);
+        const bool check = --ncheck == 0 || it == a.max_iter;
+        if (ncheck == 0) ncheck = a.check_every;
         const int par = it & 1;
-        const bool cold = sm.flags[0] != 0.0;
-        const double mu_div = sm.flags[1];
         double cm_r = 0.0, cm_s = 0.0;
-        float fcr_all = 0.0f, fcs_all = 0.0f;
+        float fcr = 0.0f, fcs = 0.0f;
         Iter64 ic;
         if constexpr (!MIXED) {
-            ic.rho3h = 0.5 * sm.rho[2];
-            ic.rho4h = 0.5 * sm.rho[3];
-            ic.hr1 = 0.5 * sm.rho[0];
-            ic.hr1f = f64_to_f32_int(ic.hr1);
+            ic.rho3h = sm.bc[4];
+            ic.rho4h = sm.bc[5];
+            ic.hr1 = sm.bc[6];
+            ic.hr1f = fp[3];
             ic.iq = iq64;
             ic.iqh = 0.5 * iq64;
         }
@@ -478,11 +551,13 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
         // pass every row segment gets its own warps, so its segments run
         // concurrently and one reduction barrier closes them all.
         for (int jb = jf; jb <= jl; jb += prows) {
-            const SegPlan sp = seg_plan<NWP>(c0, c1, rs, jb, min(jl, jb + prows - 1), threadIdx.x >> 5);
+            const int ns = min(jl, jb + prows - 1) - jb + 1;
+            if (jb > jf) __syncthreads(); // the previous pass has been reduced
+            const SegPlan sp = jb == jf ? sp0 : seg_plan<NWP>(c0, c1, rs, jb, jb + ns - 1, threadIdx.x >> 5);
             const int j = sp.j;
-            double *rec = seg_record(a, par, j);
+            double *rec = seg_record(a, sm, par, j);
             // row-local column range of the segment (k), and this thread's start and step
-            const int kb = (int)(sp.s0 - (int64_t)j * rs), ke = (int)(sp.s1 - (int64_t)j * rs);
+            const int kb = sp.kb, ke = sp.ke;
             const int first = sp.lw * 32 + (threadIdx.x & 31), stride = sp.nw * 32;
             if constexpr (!MIXED) {
                 double gs[M], dmx[M], dmn[M];
@@ -494,7 +569,7 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
                 }
                 for (int k = kb + first; k < ke; k += stride)
                     column64<M>(a, sm, ic, j, k, check, cold, mu_div, gs, dmx, dmn, cm_r, cm_s, rec);
-                flush_segments<M, NWP>(a, par, jb, gs, dmx, dmn, check, m, sp, sm);
+                flush_segments<M, NWP>(a, par, jb, ns, gs, dmx, dmn, cm_r, cm_s, check, m, sp, sm);
             } else {
                 float2 ghi[M], glo[M]; // per-lane capacity sums of the column pairs
                 float fmx[M], fmn[M];
@@ -505,9 +580,7 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
                     fmx[i] = -INFINITY;
                     fmn[i] = INFINITY;
                 }
-                const float rho1 = (float)sm.rho[0], rho3 = (float)sm.rho[2], rho4 = (float)sm.rho[3];
-                const float iq = 1.0f / (float)q;
-                float fcr = 0.0f, fcs = 0.0f;
+                const float rho1 = fp[0], rho3 = fp[1], rho4 = fp[2], mudf = f64_to_f32_int(mu_div);
                 const ElemF32 ea = {(const float *)a.f2, (const float *)a.f1, (const float *)a.g2,
                                     (const float *)a.g1, (const float *)a.g0, (const float *)a.lo,
                                     (const float *)a.hi, (const float *)a.y,  (float *)a.x,
@@ -527,7 +600,7 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
                     for (int k0 = k00; k0 < kn; k0 += stride * VW) {
                         const int k0n = k0 + stride * VW < kn ? k0 + stride * VW : -1;
                         vec32<M, VW, PREC == ADMM_MIXED_FP64CUBIC, STAGE_ROLL>(
-                            ea, sm.uoff, sm.x1nu, j, k0, check, cold, (float)mu_div, rho1, rho3, rho4, iq, ghi, glo,
+                            ea, sm.uoff, sm.x1nu, j, k0, check, cold, mudf, rho1, rho3, rho4, iq, ghi, glo,
                             fmx, fmn, fcr, fcs, esc, rec, stw, k0n);
                     }
                     cp_async_wait0();
@@ -536,142 +609,187 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
                         if constexpr (MINB == 2) // several vectors per thread: fetch the next one into L2
                             if (k0 + stride * VW < kn) prefetch_vec32<M>(ea, j, k0 + stride * VW, cold);
                         vec32<M, VW, PREC == ADMM_MIXED_FP64CUBIC>(ea, sm.uoff, sm.x1nu, j, k0, check, cold,
-                                                                   (float)mu_div, rho1, rho3, rho4, iq, ghi, glo,
+                                                                   mudf, rho1, rho3, rho4, iq, ghi, glo,
                                                                    fmx, fmn, fcr, fcs, esc, rec);
                     }
                 }
-                fcr_all = fmaxf(fcr_all, fcr);
-                fcs_all = fmaxf(fcs_all, fcs);
-                flush_segments32<M, NWP>(a, par, jb, ghi, glo, fmx, fmn, check, m, sp, sm);
+                flush_segments32<M, NWP>(a, par, jb, ns, ghi, glo, fmx, fmn, fcr, fcs, check, m, sp, sm);
             }
         }
-        if (MIXED) {
-            cm_r = (double)fcr_all;
-            cm_s = (double)fcs_all;
-        }
-        if (check) {
-            double v[2] = {cm_r, cm_s};
-            block_max<2, NWP>(v, sm);
-            if (threadIdx.x == 0) {
-                a.cpart[((size_t)par * a.grid + blockIdx.x) * 4 + 0] = v[0];
-                a.cpart[((size_t)par * a.grid + blockIdx.x) * 4 + 1] = v[1];
+        if (check && threadIdx.x == 0) { // the CTA's column maxima (the last pass holds the largest so far)
+            double v0 = 0.0, v1 = 0.0;
+            for (int w = 0; w < NWP; ++w) {
+                v0 = max_nonneg(v0, sm.mx[w * 8]);
+                v1 = max_nonneg(v1, sm.mx[w * 8 + 1]);
             }
+            a.cpart[((size_t)par * a.grid + blockIdx.x) * 4 + 0] = v0;
+            a.cpart[((size_t)par * a.grid + blockIdx.x) * 4 + 1] = v1;
         }
         ++nbar;
         if (!grid_barrier(a.bar, nbar * (unsigned)a.grid, a.status, a.spin_ns, ADMM_ETIMEOUT)) {
             ok = false;
             break;
         }
-        if (threadIdx.x == 0) sm.flags[1] = 1.0; // the pending mu rescale has been applied
+        cold = false;
+        mu_div = 1.0; // the pending mu rescale has been applied
 
         // ---- phase 2: per-(i, j) scalar steps, redundantly in every CTA ---
-        const double rho1 = sm.rho[0], rho2 = sm.rho[1], rho3 = sm.rho[2];
-        double r2m = 0.0, r3m = 0.0, s1m = 0.0, s2m = 0.0;
-        for (int pr = threadIdx.x; pr < mq; pr += NT) {
+        // Two independent chains on different warps: the mean over j of step (c)
+        // with (h), one warp per source from the last warp down, and steps (b),
+        // (d), (g), (i) per pair, G lanes sharing a pair's records; one CTA barrier
+        // closes both.  Bound by latency: the records' L2 round trip and a chain
+        // of about 15 FP64 instructions of 64 cycles.  With the reductions above,
+        // per iteration (us): n = 1000, q = 50 PHEV FP64 16.7 -> 12.1, mixed
+        // 10.0 -> 7.7; n = 4099, m = 3, q = 7 FP64 23.3 -> 15.2; n = 10007, m = 6,
+        // q = 11 mixed 31.4 -> 24.0; n = 100 FP64 1.8x.
+        const size_t rstride = (size_t)m * 4;
+        const double *prec = a.part + (size_t)par * q * a.nbmax * rstride;
+        double r1m = 0.0, r2m = 0.0, r3m = 0.0, r4m = 0.0, s1m = 0.0, s2m = 0.0, s3m = 0.0;
+        {
+            const int i = NWP - 1 - (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
+            if (i < m) {
+                double sum = 0.0;
+                for (int j = lane; j < q; j += 32) {
+                    // x at k = 0: FP64 in the FP64 kernel, FP32 in the first four bytes of the slot in the mixed ones
+                    const double *r0 = prec + (size_t)j * a.nbmax * rstride + i * 4 + 3;
+                    const double x0 = MIXED ? f32_to_f64_int(__ldcg((const float *)r0)) : ldcg(r0);
+                    const double d = x0 - sm.nu[i * q + j];
+                    sm.x0[i * q + j] = x0;
+                    sum = j == lane ? d : sum + d;
+                }
+                const double x1n = warp_sum(sum) * iq64;              // (c), the mean over j
+                for (int j = lane; j < q; j += 32) {
+                    const int pr = i * q + j;
+                    const double d = x1n - sm.x0[pr], nun = sm.nu[pr] + d; // (h)
+                    sm.nu[pr] = nun;
+                    if (MIXED) sm.x1nu[pr] = f64_to_f32_int(x1n + nun);
+                    if (check) r4m = max_nonneg(r4m, fabs(d));
+                }
+                if (lane == 0) sm.x1[i] = x1n;
+            }
+        }
+        const double kappa = sm.bc[3];
+        for (int p0 = 0; p0 < mq; p0 += NT >> gsh) {
+            if (p0 + (int)((threadIdx.x & ~31u) >> gsh) >= mq) break; // the whole warp is past the pairs
+            const int pq = p0 + (int)(threadIdx.x >> gsh), sub = threadIdx.x & (G - 1);
+            const bool in = pq < mq;
+            const int pr = in ? pq : mq - 1;
             const int i = pr / q, j = pr - i * q;
-            const int nb = row_ctas(a, j);
-            const double *rec = a.part + ((size_t)(par * q + j) * a.nbmax) * m * 4 + i * 4;
-            const int stride = m * 4;
-            // records of row j, in CTA order; independent loads, fixed order of the sums
+            const int nb = sm.rcnt[j];
+            const double *rec = prec + (size_t)j * a.nbmax * rstride + i * 4;
+            const double g0s = a.sumg0[pr], ci = a.c[i];
+            // records of row j in CTA order, every G-th per lane; a fixed order of the sums
             double S = 0.0, dmx = -INFINITY, dmn = INFINITY;
-            // x at k = 0: FP64 in the FP64 kernel, FP32 in the first four bytes of the slot in the mixed ones
-            const double x0 = MIXED ? (double)__ldcg((const float *)(rec + 3)) : ldcg(rec + 3);
 #pragma unroll 8
-            for (int t = 0; t < nb; ++t) {
-                S += ldcg(rec + (size_t)t * stride);
+            for (int t = sub; t < nb; t += G) {
+                const double v = ldcg(rec + (size_t)t * rstride);
+                S = t == sub ? v : S + v;
                 if (check) {
-                    dmx = fmax(dmx, ldcg(rec + (size_t)t * stride + 1));
-                    dmn = fmin(dmn, ldcg(rec + (size_t)t * stride + 2));
+                    dmx = max_ord(dmx, ldcg(rec + (size_t)t * rstride + 1));
+                    dmn = min_ord(dmn, ldcg(rec + (size_t)t * rstride + 2));
+                }
+            }
+            for (int o = G >> 1; o > 0; o >>= 1) {
+                S += __shfl_xor_sync(0xffffffffu, S, o);
+                if (check) {
+                    dmx = max_ord(dmx, __shfl_xor_sync(0xffffffffu, dmx, o));
+                    dmn = min_ord(dmn, __shfl_xor_sync(0xffffffffu, dmn, o));
                 }
             }
             const double lam = sm.lam[pr], zeta = sm.zeta[pr], hh = sm.h[pr], pp = sm.p[pr];
-            const double W = (S + a.sumg0[pr]) - (double)n * lam;     // 1'(g(x) - lambda)
+            const double W = fma(-nd, lam, S + g0s);                  // 1'(g(x) - lambda)
             const double lamn = kappa * ((hh + pp) - W);              // (b) + (g)
-            const double Z = W + (double)n * lamn;                    // 1'z
-            const double cz = Z - pp;
-            const double hn = cz < a.c[i] ? cz : a.c[i];              // (d)
-            const double pn = pp + (hn - Z);                          // (i)
-            if (check) {
-                r2m = max_nonneg(r2m, fabs(lamn - lam));
-                r3m = max_nonneg(r3m, fabs(hn - Z));
-                const double dl = (lamn - lam) - zeta;
+            const double Z = fma(nd, lamn, W);                        // 1'z
+            const double hn = min_ord(Z - pp, ci);                    // (d)
+            const double e = hn - Z, zn = lamn - lam;
+            if (check && in) { // a lane past the pairs may see the last pair's new scalars
+                r2m = max_nonneg(r2m, fabs(zn));
+                r3m = max_nonneg(r3m, fabs(e));
+                const double dl = zn - zeta;
                 s1m = max_nonneg(s1m, max_nonneg(fabs(dmx + dl), fabs(dmn + dl)));
                 s2m = max_nonneg(s2m, fabs(hn - hh));
             }
-            sm.lam[pr] = lamn;
-            sm.zeta[pr] = lamn - lam;
-            sm.h[pr] = hn;
-            sm.p[pr] = pn;
-            sm.x0[pr] = x0;
-        }
-        __syncthreads();
-        for (int i = threadIdx.x >> 5; i < m; i += NWP) {        // (c), mean over j: warp i, source i
-            const int lane = threadIdx.x & 31;
-            double sum = 0.0;
-            for (int j = lane; j < q; j += 32) sum += sm.x0[i * q + j] - sm.nu[i * q + j];
-            sum = warp_sum(sum);
-            if (lane == 0) sm.x1n[i] = sum / (double)q;
-        }
-        __syncthreads();
-        double r4m = 0.0;
-        for (int pr = threadIdx.x; pr < mq; pr += NT) {          // (h)
-            const int i = pr / q;
-            const double x0 = sm.x0[pr], x1n = sm.x1n[i];
-            sm.nu[pr] = sm.nu[pr] + (x1n - x0);
-            if (check) r4m = max_nonneg(r4m, fabs(x0 - x1n));
-        }
-        __syncthreads();
-        if (threadIdx.x < m) sm.x1[threadIdx.x] = sm.x1n[threadIdx.x];
-        if (threadIdx.x == 0) sm.flags[0] = 0.0;
-        __syncthreads();
-
-        if (check) {
-            double r1 = 0.0, s3 = 0.0;
-            for (int b = threadIdx.x; b < a.grid; b += NT) {
-                r1 = max_nonneg(r1, ldcg(a.cpart + ((size_t)par * a.grid + b) * 4 + 0));
-                s3 = max_nonneg(s3, ldcg(a.cpart + ((size_t)par * a.grid + b) * 4 + 1));
+            __syncwarp(); // the lanes of a pair have read its scalars
+            if (in && sub == 0) {
+                sm.lam[pr] = lamn;
+                sm.zeta[pr] = zn;
+                sm.h[pr] = hn;
+                sm.p[pr] = pp + e;                                    // (i)
+                if (MIXED) sm.uoff[pr] = f64_to_f32_int(zn + lamn);
+                else sm.zl[pr] = zn + lamn;
             }
-            double v[7] = {r1, r2m, r3m, r4m, s1m, s2m, s3};
-            block_max<7, NWP>(v, sm);
+        }
+        if (check) { // maxima over the CTA, and over the CTAs' columns
+            for (int b = threadIdx.x; b < a.grid; b += NT) {
+                r1m = max_nonneg(r1m, ldcg(a.cpart + ((size_t)par * a.grid + b) * 4 + 0));
+                s3m = max_nonneg(s3m, ldcg(a.cpart + ((size_t)par * a.grid + b) * 4 + 1));
+            }
+            double v[8] = {r1m, r2m, r3m, r4m, s1m, s2m, s3m, 0.0};
+            auto mx = [](double k, double s, int o) { return max_nonneg(k, __shfl_xor_sync(0xffffffffu, s, o)); };
+            const double r = warp_many<8>(v, mx);
+            if ((threadIdx.x & 3) == 0) sm.mx[(threadIdx.x >> 5) * 8 + ((threadIdx.x & 31) >> 2)] = r;
+        }
+        __syncthreads();
+        if (check) {
+            // thread 0 takes the stop decision and the adaptation of Sec. IV-A and passes them on
+            int *dec = (int *)(sm.bc + 7);
+            if (threadIdx.x == 0) {
+                double v[7];
 #pragma unroll
-            for (int t = 0; t < 7; ++t) res[t] = v[t];
-            const double r = fmax(fmax(v[0], v[1]), fmax(v[2], v[3]));
-            const double sg = fmax(fmax(rho1 * v[4], rho2 * v[5]), rho3 * v[6]);
-            r_last = r;
-            s_last = sg;
-            if (r < a.r_tol && sg < a.s_tol) {
+                for (int t = 0; t < 7; ++t) {
+                    v[t] = 0.0;
+                    for (int w = 0; w < NWP; ++w) v[t] = max_nonneg(v[t], sm.mx[w * 8 + t]);
+                    res[t] = v[t];
+                }
+                const double r = max_nonneg(max_nonneg(v[0], v[1]), max_nonneg(v[2], v[3]));
+                const double sg = max_nonneg(max_nonneg(sm.rho[0] * v[4], sm.rho[1] * v[5]), sm.rho[2] * v[6]);
+                r_last = r;
+                s_last = sg;
+                const bool cv = r < a.r_tol && sg < a.s_tol;
+                double f = 1.0;
+                if (!cv && a.adapt && it < a.max_iter && it >= a.adapt_start) { // Sec. IV-A, duals rescaled
+                    const double ratio = r / sg, target = a.adapt_target;
+                    if (ratio > 1.2 * target) f = a.tau;
+                    else if (ratio < 0.8 * target) f = 1.0 / a.tau;
+                }
+                dec[0] = cv;
+                dec[1] = f != 1.0;
+                sm.bc[2] = f;
+                if (f != 1.0) {
+                    for (int t = 0; t < 4; ++t) sm.rho[t] *= f;
+                    derive_penalties(sm, n);
+                }
+            }
+            __syncthreads();
+            if (dec[0]) {
                 conv = true;
                 break;
             }
-            if (a.adapt && it < a.max_iter && it >= a.adapt_start) { // Sec. IV-A, duals rescaled
-                const double ratio = r / sg, target = a.adapt_target;
-                double f = 1.0;
-                if (ratio > 1.2 * target) f = a.tau;
-                else if (ratio < 0.8 * target) f = 1.0 / a.tau;
-                if (f != 1.0) {
-                    for (int pr = threadIdx.x; pr < mq; pr += NT) {
-                        sm.lam[pr] /= f;
-                        sm.p[pr] /= f;
-                        sm.nu[pr] /= f;
+            if (dec[1]) {
+                const double f = sm.bc[2];
+                for (int pr = threadIdx.x; pr < mq; pr += NT) {
+                    const double l = sm.lam[pr] / f, nu = sm.nu[pr] / f;
+                    sm.lam[pr] = l;
+                    sm.p[pr] /= f;
+                    sm.nu[pr] = nu;
+                    if (MIXED) {
+                        sm.uoff[pr] = (float)(sm.zeta[pr] + l);
+                        sm.x1nu[pr] = (float)(sm.x1[pr / q] + nu);
+                    } else {
+                        sm.zl[pr] = sm.zeta[pr] + l;
                     }
-                    __syncthreads();
-                    if (threadIdx.x < 4) sm.rho[threadIdx.x] *= f;
-                    if (threadIdx.x == 0) sm.flags[1] = f;
-                    __syncthreads();
-                    kappa = sm.rho[1] / (sm.rho[0] + (double)n * sm.rho[1]);
                 }
+                mu_div = f;
+                __syncthreads();
             }
         }
-        for (int pr = threadIdx.x; pr < mq; pr += NT) {
-            if constexpr (MIXED) {
-                sm.uoff[pr] = (float)(sm.zeta[pr] + sm.lam[pr]);
-                sm.x1nu[pr] = (float)(sm.x1[pr / q] + sm.nu[pr]);
-            } else {
-                sm.zl[pr] = sm.zeta[pr] + sm.lam[pr];
-            }
-        }
-        __syncthreads();
     }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        sm.flags[0] = cold ? 1.0 : 0.0;
+        sm.flags[1] = mu_div;
+    }
+    __syncthreads();
     const int iters = it > a.max_iter ? a.max_iter : it;
 
     // ---- objective (1/q) sum f(x) of eq. (2): one more barrier -----------
