@@ -31,13 +31,11 @@ namespace admm_impl {
 // only on the coefficients), and the discriminant bound below allows for a
 // reciprocal that is off by 2 ulp.
 __device__ __forceinline__ float rcp_fast(float v) { return __fdividef(1.0f, v); }
+__device__ __forceinline__ float rsqrt_fast(float v) { return rsqrtf(v); }
 __device__ __forceinline__ float sqrt_fast(float v) { return v > 0.0f ? v * rsqrtf(v) : 0.0f; }
-__device__ __forceinline__ float cbrt_fast(float v)
-{
-    const float a = fabsf(v);
-    const float r = a > 0.0f ? exp2f(__log2f(a) * (1.0f / 3.0f)) : 0.0f;
-    return copysignf(r, v);
-}
+// |v|^(1/3) for v != 0
+__device__ __forceinline__ float cbrt_abs(float v) { return exp2f(__log2f(fabsf(v)) * (1.0f / 3.0f)); }
+__device__ __forceinline__ float cbrt_fast(float v) { return copysignf(v != 0.0f ? cbrt_abs(v) : 0.0f, v); }
 
 // The FP64 closed form, out of line: taken only when FP32 overflows.
 static __device__ __noinline__ float quartic_min_fallback64(float A, float B, float C, float D, float lo, float hi,
@@ -157,7 +155,7 @@ __device__ __forceinline__ float quartic_min32(float A, float B, float C, float 
     if (branch == 1) return clampf(-b3, lo, hi);
     if (branch == 0) {
         // Delta > 0 here (certified, or FP64 said so): as in the packed path
-        const float sq = Dl > 0.0f ? __fmul_rn(Dl, rsqrtf(Dl)) : 0.0f;
+        const float sq = Dl > 0.0f ? __fmul_rn(Dl, rsqrt_fast(Dl)) : 0.0f;
         const float S = cbrt_fast(__fadd_rn(R, R >= 0.0f ? sq : -sq));
         const float T = S != 0.0f ? __fmul_rn(-Q, rcp_fast(S)) : 0.0f;
         const float x = newton_polish32(A, B, C, D, __fsub_rn(__fadd_rn(S, T), b3));
@@ -184,22 +182,62 @@ __device__ __forceinline__ float quartic_min32(float A, float B, float C, float 
     return delta_f32(u, v, b, c, d) > 0.0f ? v : u;
 }
 
+// cos(acos(a) / 3) for a in [-1, 1], whose 2 sqrt(-Q)-fold is the largest
+// root of z^3 + 3 Q z - 2 R with a = R / sqrt(-Q)^3 (and, of -a, minus the
+// smallest): with w = sqrt((1 + a) / 2) = cos(acos(a) / 2) it is
+// cos((2/3) acos w), analytic on [0, 1] (the nearest singularity is w = -1), here
+// by its degree-7 Chebyshev interpolant (error 1e-7 in FP32 arithmetic).
+__device__ __forceinline__ float sqrt_approx(float v)
+{
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+#define ADMM_THIRD_COEFS                                                                                   \
+    {0.5f, 0.577347219f, -0.111043237f, 0.0528691076f, -0.0303130634f, 0.0161594898f, -0.00616994966f, 0.00115042902f}
+__device__ __forceinline__ float cos_third(float a)
+{
+    const float k[8] = ADMM_THIRD_COEFS;
+    const float w = sqrt_approx(fmaf(0.5f, a, 0.5f));
+    float r = k[7];
+#pragma unroll
+    for (int t = 6; t >= 0; --t) r = fmaf(r, w, k[t]);
+    return r;
+}
+
+// Newton step and slope of the derivative's half H(x) = 2A x^3 + 1.5B x^2 + C x + D/2 in FP32.
+__device__ __forceinline__ void half_polish32(float A2, float B15, float C, float Dh, float &x, float &s)
+{
+    const float h = fmaf(fmaf(fmaf(A2, x, B15), x, C), x, Dh);
+    const float sl = fmaf(fmaf(3.0f * A2, x, 2.0f * B15), x, C);
+    const float dx = h * rcp_fast(sl);
+    if (sl > 0.0f && fabsf(dx) <= 0.0625f * (fabsf(x) + 1.0f)) x -= dx;
+    s = fmaf(fmaf(3.0f * A2, x, 2.0f * B15), x, C);
+}
+
 // ---------------------------------------------------------------------------
 // FP64 minimiser seeded in FP32.  FP64 throughput is 1/64 of FP32 on this
-// GPU, so for the Cardano branch the root is found in FP32 (closed form +
-// Newton step, as in quartic_min32) and then refined by two FP64 Newton steps
-// on the FP64 derivative 4A x^3 + 3B x^2 + 2C x + D (step divisor from an
-// FP32 reciprocal: each step multiplies the relative error by about the
-// FP32 unit roundoff, so two steps reach FP64 rounding).  The FP32 branch
-// test is certified against the FP64 coefficients: the error bound of
-// quartic_min32 is doubled for the rounding of A, B, C, D to FP32.  Anything
-// else (quadratic, trig or uncertain branch, FP32 range, a step that did not
-// settle) takes the FP64 closed form of quartic_min64.
+// GPU, so everything that can be decided in FP32 with certainty is: the
+// branch of the cubic (the error bound of quartic_min32, doubled for the
+// rounding of A, B, C, D to FP32), and on the trig branch which of the two
+// minima is the constrained minimiser (the sign of F(u) - F(v) = (u - v) br
+// where |br| exceeds 1e-5 of the sum of its terms' magnitudes; FP32 makes an
+// error of a few 1e-7 of it).  Only the chosen root is refined, by two FP64
+// Newton steps on half the derivative with one FP32 slope: 9 FP64-pipe
+// instructions in all, where both closed forms took 186 per warp.  Anything
+// uncertain, out of the FP32 range, or not settled takes the FP64 closed form.
+// 1e6 quartics (a third of them double wells): 571 -> 43 us a call on device arrays (kernel 381 -> 29 us).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ bool cardano_seed32(double A64, double B64, double C64, double D64, float &root)
+static __device__ __noinline__ double quartic_min64_closed(double A, double B, double C, double D, double lo,
+                                                           double hi, int paper_mode)
 {
-    const float A = (float)A64, B = (float)B64, C = (float)C64, D = (float)D64;
-    if (!(A > 1.0e-30f && A < 1.0e30f)) return false;
+    return quartic_min64(A, B, C, D, lo, hi, paper_mode);
+}
+
+// FP32 root to refine (x) and the slope of H there (s); false: not certain.
+__device__ __forceinline__ bool quartic_seed32(float A, float B, float C, float D, float lo, float hi,
+                                               int paper_mode, float &x, float &s)
+{
     const float inv = rcp_fast(A);
     const float b = 0.75f * B * inv, c = 0.5f * C * inv, d = 0.25f * D * inv;
     const float b3 = b * (1.0f / 3.0f);
@@ -210,31 +248,85 @@ __device__ __forceinline__ bool cardano_seed32(double A64, double B64, double C6
     const float mQ = fabsf(c) * (1.0f / 3.0f) + b3 * b3;
     const float mR = fabsf(b3 * 0.5f * c) + fabsf(b3 * b3 * b3) + 0.5f * fabsf(d);
     const float bound = 1.2e-7f * (96.0f * Q * Q * mQ + 64.0f * fabsf(Q3) + 96.0f * fabsf(R) * mR + 64.0f * R2);
-    if (!(Dl > bound)) return false;
-    const float sq = sqrt_fast(Dl);
-    const float S = cbrt_fast(R >= 0.0f ? R + sq : R - sq);
-    const float T = S != 0.0f ? -Q * rcp_fast(S) : 0.0f;
-    root = newton_polish32(A, B, C, D, S + T - b3);
-    return isfinite(root);
+    const float A2 = A + A, B15 = 1.5f * B, Dh = 0.5f * D;
+    if (Dl > bound) {
+        const float sq = sqrt_fast(Dl);
+        const float S = cbrt_fast(R >= 0.0f ? R + sq : R - sq);
+        x = S - Q * rcp_fast(S) - b3;
+        half_polish32(A2, B15, C, Dh, x, s);
+        return true;
+    }
+    if (!(Dl < -bound)) return false;
+    const float rs = rsqrt_fast(-Q), sq2 = 2.0f * -Q * rs;
+    const float arg = fminf(fmaxf(R * (rs * rs * rs), -1.0f), 1.0f);
+    float x3 = fmaf(sq2, cos_third(arg), -b3), x1 = fmaf(-sq2, cos_third(-arg), -b3), s1, s3;
+    half_polish32(A2, B15, C, Dh, x1, s1);
+    half_polish32(A2, B15, C, Dh, x3, s3);
+    float u = x1, v = x3;
+    bool third = false;
+    if (!paper_mode) {
+        u = clampf(x1, lo, hi);
+        v = clampf(x3, lo, hi);
+        // both minima on one side of the interval: the same end of it
+        if (x3 < lo - 1.0e-5f * (fabsf(lo) + 1.0f) || x1 > hi + 1.0e-5f * (fabsf(hi) + 1.0f)) u = v;
+        else if (!(v - u > 1.0e-4f * (fabsf(u) + fabsf(v) + 1.0f))) return false;
+    }
+    if (u != v) {
+        const float uu = u * u, vv = v * v, uv = u * v;
+        const float t3 = A * (u + v) * (uu + vv), t2 = B * (uu + uv + vv), t1 = C * (u + v); // u^3 + u^2 v + u v^2 + v^3
+        const float m3 = A * (fabsf(u) + fabsf(v)) * (uu + vv), m2 = fabsf(B) * (uu + fabsf(uv) + vv),
+                    m1 = fabsf(C) * (fabsf(u) + fabsf(v));
+        const float br = t3 + t2 + t1 + D;
+        if (!(fabsf(br) > 1.0e-5f * (m3 + m2 + m1 + fabsf(D)))) return false;
+        third = br < 0.0f; // u < v: F(u) > F(v)
+    }
+    x = third ? x3 : x1;
+    s = third ? s3 : s1;
+    return true;
 }
 
+// v / 2 on the integer pipes (a denormal result gives a signed zero)
+__device__ __forceinline__ double half64(double v)
+{
+    const int h = __double2hiint(v);
+    const bool z = (h & 0x7ff00000) <= 0x00100000;
+    return __hiloint2double(z ? h & 0x80000000 : h - 0x00100000, z ? 0 : __double2loint(v));
+}
+
+__device__ __forceinline__ bool newton_settled(float d0, float d1, float x);
+
+// Called by whole warps: the lanes come together again before the FP64
+// refinement, which a warp with several branches would otherwise run once for each
+// (30 FP64 instructions per warp instead of 10).
 __device__ __forceinline__ double quartic_min64_seeded(double A, double B, double C, double D, double lo, double hi,
                                                        int paper_mode)
 {
-    float r32;
-    if (A != 0.0 && cardano_seed32(A, B, C, D, r32)) {
-        const double A4 = 4.0 * A, B3 = 3.0 * B, C2 = 2.0 * C, A12 = 12.0 * A, B6 = 6.0 * B;
-        double x = (double)r32, step = 0.0;
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            const double p = ((A4 * x + B3) * x + C2) * x + D;
-            const double pp = (A12 * x + B6) * x + C2;
-            step = p * (double)rcp_approx_f32((float)pp);
-            x -= step;
-        }
-        if (fabs(step) <= 1.0e-12 * (fabs(x) + 1.0)) return clampd(x, lo, hi);
+    const bool lin = (__double_as_longlong(A) << 1) == 0; // A = 0: B plays no part
+    const float Af = f64_to_f32_int(A), Cf = f64_to_f32_int(C), Df = f64_to_f32_int(D);
+    float xf = 0.0f, sf = 0.0f;
+    if (lin) {
+        xf = -0.5f * Df * rcp_fast(Cf);
+        sf = Cf;
+    } else if (Af > 1.0e-30f && Af < 1.0e30f) {
+        if (!quartic_seed32(Af, f64_to_f32_int(B), Cf, Df, f64_to_f32_int(lo), f64_to_f32_int(hi), paper_mode, xf, sf))
+            sf = 0.0f;
     }
-    return quartic_min64(A, B, C, D, lo, hi, paper_mode);
+    __syncwarp();
+    const float rf = rcp_fast(sf);
+    // A lies in the FP32 range, so doubling it is one more in the exponent
+    const double A2 = lin ? 0.0 : __longlong_as_double(__double_as_longlong(A) + 0x0010000000000000ll);
+    const double B15 = lin ? 0.0 : 1.5 * B, Dh = half64(D), r = f32_to_f64_int(rf);
+    double x = f32_to_f64_int(xf);
+    float dn[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        const double H = fma(fma(fma(A2, x, B15), x, C), x, Dh);
+        x = fma(-H, r, x);
+        dn[t] = f64_to_f32_int(H) * rf;
+    }
+    if (sf > 0.0f && isfinite(xf) && isfinite(rf) && rf >= 1.2e-38f && newton_settled(dn[0], dn[1], xf))
+        return clamp_ord(x, lo, hi);
+    return quartic_min64_closed(A, B, C, D, lo, hi, paper_mode);
 }
 
 // ---------------------------------------------------------------------------
@@ -292,7 +384,7 @@ __device__ __forceinline__ bool elem_polish32(float b2, float b1, float u, float
 static __device__ __noinline__ bool elem_trig32(float Q, float R, float dR, float b3, float lo, float hi,
                                                 int paper_mode, float &y)
 {
-    const float nQ = -Q, s = sqrt_fast(nQ);
+    const float nQ = -Q, s = sqrt_fast(nQ); // nQ > 0: Delta < 0 is certified
     const float mlo = 1.0e-5f * (fabsf(lo) + fabsf(b3) + 1.0f), mhi = 1.0e-5f * (fabsf(hi) + fabsf(b3) + 1.0f);
     int side = 0;
     if (!paper_mode) {
@@ -305,7 +397,8 @@ static __device__ __noinline__ bool elem_trig32(float Q, float R, float dR, floa
         side = R > 0.0f ? 1 : -1;
     }
     const float Rs = side > 0 ? R : -R;
-    const float arg = fminf(fmaxf(Rs * rsqrtf(nQ * nQ * nQ), -1.0f), 1.0f);
+    const float rs = rsqrt_fast(nQ);
+    const float arg = fminf(fmaxf(Rs * (rs * rs * rs), -1.0f), 1.0f);
     const float z = 2.0f * s * __cosf(acosf(arg) * (1.0f / 3.0f));
     y = (side > 0 ? z : -z) - b3;
     return basin || paper_mode || (y > lo + mlo && y < hi - mhi);
@@ -459,10 +552,9 @@ __device__ __forceinline__ float2 quartic_min32x2(float2 A, float2 B, float2 C, 
             // here Delta > bound >= 0, so sqrt(Delta) > 0, |R +- sqrt(Delta)| > 0 and S != 0: the
             // zero guards of sqrt_fast, cbrt_fast and the T reciprocal are not needed (an S that
             // underflows gives a non-finite x and the lane-by-lane path below)
-            const float2 sq = mul2(Dl, make_float2(rsqrtf(Dl.x), rsqrtf(Dl.y)));
+            const float2 sq = mul2(Dl, make_float2(rsqrt_fast(Dl.x), rsqrt_fast(Dl.y)));
             const float2 v = add2(R, make_float2(R.x >= 0.0f ? sq.x : -sq.x, R.y >= 0.0f ? sq.y : -sq.y));
-            const float2 S = make_float2(copysignf(exp2f(__log2f(fabsf(v.x)) * (1.0f / 3.0f)), v.x),
-                                         copysignf(exp2f(__log2f(fabsf(v.y)) * (1.0f / 3.0f)), v.y));
+            const float2 S = make_float2(copysignf(cbrt_abs(v.x), v.x), copysignf(cbrt_abs(v.y), v.y));
             const float2 rS = make_float2(rcp_fast(S.x), rcp_fast(S.y));
             const float2 T = mul2(neg2(Q), rS);
             const float2 x = newton_polish32x2(A, B, C, D, sub2(add2(S, T), b3));
@@ -477,6 +569,96 @@ __device__ __forceinline__ float2 quartic_min32x2(float2 A, float2 B, float2 C, 
     }
 #endif
     return quartic_min32_lanes(A, B, C, D, lo, hi, paper_mode, &esc);
+}
+
+// The same for many quartics with any mix of single and double wells (the
+// quartic benchmark, where a third are double wells and nearly every warp holds
+// both branches): both lanes' Cardano root and both lanes' trig roots are found
+// packed, and each lane keeps what its branch needs, instead of one lane after
+// the other through the scalar code (725 -> 347 warp instructions per 64
+// quartics).  The decisions are those of quartic_min32: the branch outside
+// its error bound, the lower minimum where |br| of F(u) - F(v) = (u - v) br
+// exceeds 2e-5 of the sum of its terms' magnitudes (FP32 errs by a few 1e-7
+// of it).  A pair with anything nearer than that, A = 0, or a value that is
+// not finite goes through quartic_min32_lanes.
+__device__ __forceinline__ float2 min2(float2 a, float2 b) { return make_float2(fminf(a.x, b.x), fminf(a.y, b.y)); }
+__device__ __forceinline__ float2 max2(float2 a, float2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
+__device__ __forceinline__ float2 sel2(bool px, bool py, float2 a, float2 b)
+{
+    return make_float2(px ? a.x : b.x, py ? a.y : b.y);
+}
+__device__ __forceinline__ float2 cos_third2(float2 a)
+{
+    const float2 h = fma2(splat2(0.5f), a, splat2(0.5f));
+    const float2 w = make_float2(sqrt_approx(h.x), sqrt_approx(h.y));
+    const float k[8] = ADMM_THIRD_COEFS;
+    float2 r = splat2(k[7]);
+#pragma unroll
+    for (int t = 6; t >= 0; --t) r = fma2(r, w, splat2(k[t]));
+    return r;
+}
+
+__device__ __forceinline__ float2 quartic_min32x2_wells(float2 A, float2 B, float2 C, float2 D, float2 lo, float2 hi,
+                                                        int paper_mode, unsigned &esc)
+{
+    const float2 inv = make_float2(rcp_fast(A.x), rcp_fast(A.y));
+    const float2 b = mul2(mul2(splat2(0.75f), B), inv);
+    const float2 c = mul2(mul2(splat2(0.5f), C), inv);
+    const float2 d = mul2(mul2(splat2(0.25f), D), inv);
+    const float2 b3 = mul2(b, splat2(1.0f / 3.0f));
+    const float2 b3s = mul2(b3, b3);
+    const float2 nQ = fma2(c, splat2(-1.0f / 3.0f), b3s); // -Q
+    const float2 hc = mul2(splat2(0.5f), c), hd = mul2(splat2(0.5f), d);
+    const float2 R = sub2(sub2(mul2(b3, hc), mul2(b3s, b3)), hd);
+    const float2 Qs = mul2(nQ, nQ);
+    const float2 Dl = sub2(mul2(R, R), mul2(Qs, nQ));
+    // the forward error bound of quartic_min32, on both lanes
+    const float2 ahc = abs2(hc), ahd = abs2(hd);
+    const float2 mQ = fma2(ahc, splat2(2.0f / 3.0f), b3s);
+    const float2 mR = fma2(abs2(b3), add2(b3s, ahc), ahd);
+    const float2 bound = mul2(splat2(7.68e-6f), fma2(Qs, mQ, mul2(abs2(R), mR)));
+    const bool cx = Dl.x > bound.x, cy = Dl.y > bound.y, tx = Dl.x < -bound.x, ty = Dl.y < -bound.y;
+    bool ok = A.x > 0.0f && A.y > 0.0f && (cx || tx) && (cy || ty);
+    // sqrt(Delta) on the Cardano branch, sqrt(-Q) on the trig branch
+    const float2 rad = sel2(cx, cy, Dl, nQ);
+    const float2 rs = make_float2(rsqrt_fast(rad.x), rsqrt_fast(rad.y));
+    const float2 sq = mul2(rad, rs);
+    float2 u, v = splat2(0.0f); // Cardano: the root; trig: the smallest and the largest root
+    {
+        const float2 w = add2(R, make_float2(R.x >= 0.0f ? sq.x : -sq.x, R.y >= 0.0f ? sq.y : -sq.y));
+        const float2 S = make_float2(copysignf(cbrt_abs(w.x), w.x), copysignf(cbrt_abs(w.y), w.y));
+        u = sub2(fma2(nQ, make_float2(rcp_fast(S.x), rcp_fast(S.y)), S), b3);
+    }
+    const bool any_trig = __any_sync(__activemask(), tx || ty);
+    if (any_trig) {
+        const float2 arg = max2(min2(mul2(R, mul2(rs, mul2(rs, rs))), splat2(1.0f)), splat2(-1.0f));
+        const float2 sq2 = add2(sq, sq);
+        v = sub2(mul2(sq2, cos_third2(arg)), b3);
+        u = sel2(tx, ty, neg2(fma2(sq2, cos_third2(neg2(arg)), b3)), u);
+        v = newton_polish32x2(A, B, C, D, v);
+        v = sel2(tx, ty, v, u);
+    }
+    u = newton_polish32x2(A, B, C, D, u);
+    const float2 fin = fma2(u, splat2(0.0f), mul2(v, splat2(0.0f))); // 0 where u and v are finite, else NaN
+    ok = ok && fin.x + fin.y == 0.0f;
+    float2 x = max2(min2(u, hi), lo);
+    if (any_trig) {
+        const float2 vc = max2(min2(v, hi), lo);
+        const float2 p = paper_mode ? u : x, r = paper_mode ? v : vc;
+        const float2 s = add2(p, r), pp = mul2(p, p), rr = mul2(r, r), pr = mul2(p, r);
+        const float2 q2 = add2(pp, rr), q3 = add2(q2, pr);
+        const float2 as = add2(abs2(p), abs2(r)), b3q = mul2(b3, q3), cs = mul2(hc, s);
+        // br = (u^3 + u^2 v + u v^2 + v^3) / 4 + (b/3) (u^2 + u v + v^2) + (c/2) (u + v) + d
+        const float2 q4 = mul2(splat2(0.25f), q2);
+        const float2 br = add2(add2(fma2(q4, s, b3q), cs), d);
+        const float2 mb = add2(fma2(q4, as, abs2(b3q)), fma2(ahc, as, add2(ahd, ahd)));
+        const float2 lim = mul2(splat2(2.0e-5f), mb);
+        const bool nx = tx && p.x != r.x, ny = ty && p.y != r.y; // u < v: the larger root where br < 0
+        ok = ok && (!nx || fabsf(br.x) > lim.x) && (!ny || fabsf(br.y) > lim.y);
+        x = sel2(nx && br.x < 0.0f, ny && br.y < 0.0f, vc, x);
+    }
+    if (!ok) return quartic_min32_lanes(A, B, C, D, lo, hi, paper_mode, &esc);
+    return x;
 }
 
 } // namespace admm_impl

@@ -1,14 +1,16 @@
 // Algorithm 1 + clamp on many independent quartics (the quartic benchmark
-// of Sec. III-C): admm_quartic_min (FP64, the solver's FP64 minimiser) and
-// admm_quartic_min_f32 (FP32 on packed column pairs, the solver's mixed
-// minimiser, branch decisions as FP64 would take them).  Each thread takes
-// consecutive elements (pairs in FP32) in a grid-stride loop: 7 streams of
-// one value each, coalesced; the kernels are HBM bound once the minimiser
-// is cheap enough.  Invalid elements (A < 0, A = C = 0, lo > hi, non-finite)
-// get x = NaN and are counted.
+// of Sec. III-C): admm_quartic_min (FP64, quartic_min64_seeded) and
+// admm_quartic_min_f32 (FP32 on packed pairs, quartic_min32x2_wells, branch
+// decisions as FP64 would take them).  Each thread takes consecutive
+// elements (pairs in FP32) in a grid-stride loop: 7 streams of one value
+// each, coalesced.  Invalid elements (A < 0, A = C = 0, lo > hi, non-finite)
+// get x = NaN and are counted, per thread first, then once per block in a
+// word of pinned host memory that the call owns while it runs, so a call
+// allocates and copies nothing for it.
 #include <algorithm>
 #include <cstdint>
 #include <cstdio>
+#include <mutex>
 
 #include <cuda_runtime.h>
 
@@ -20,68 +22,145 @@ using namespace admm_impl;
 
 namespace {
 
+// Comparisons on the integer pipes: see quartic64.cuh.
 __device__ __forceinline__ bool quartic_ok(double A, double B, double C, double D, double lo, double hi)
 {
-    return isfinite(A) && isfinite(B) && isfinite(C) && isfinite(D) && !isnan(lo) && !isnan(hi) && A >= 0.0 &&
-           (A > 0.0 || C > 0.0) && lo <= hi;
+    const long long a = __double_as_longlong(A), l = __double_as_longlong(lo), h = __double_as_longlong(hi);
+    const bool zero_a = (a << 1) == 0;
+    auto top = [](double v) { return __double2hiint(v) & 0x7fffffff; }; // >= 0x7ff00000: not finite
+    auto is_nan = [](long long v) { return (unsigned long long)(v << 1) > 0xffe0000000000000ull; };
+    return max(max(top(A), top(B)), max(top(C), top(D))) < 0x7ff00000 && !is_nan(l) && !is_nan(h) &&
+           (a > 0 || (zero_a && __double_as_longlong(C) > 0)) && (ord64(lo) <= ord64(hi) || ((l | h) << 1) == 0);
+}
+__device__ __forceinline__ bool quartic_ok(float A, float B, float C, float D, float lo, float hi)
+{
+    return isfinite(A) && isfinite(B) && isfinite(C) && isfinite(D) && A >= 0.0f && (A > 0.0f || C > 0.0f) && lo <= hi;
+}
+
+// Adds a block's invalid elements to the call's word.
+__device__ __forceinline__ void report_bad(int n, int *bad)
+{
+    const int t = __syncthreads_count(n > 0); // most calls have none
+    if (t == 0) return;
+    n = __reduce_add_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0 && n > 0) atomicAdd(bad, n);
 }
 
 __global__ void __launch_bounds__(256) quartic_many_f64(const double *A, const double *B, const double *C,
                                                         const double *D, const double *lo, const double *hi,
                                                         int64_t count, int mode, double *x, int *bad)
 {
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < count;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const double a = A[t], b = B[t], c = C[t], d = D[t], l = lo[t], h = hi[t];
-        if (quartic_ok(a, b, c, d, l, h)) {
-            x[t] = quartic_min64_seeded(a, b, c, d, l, h, mode);
-        } else {
-            x[t] = NAN;
-            atomicAdd(bad, 1);
-        }
-    }
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const bool in = t < count;
+    const int64_t u = in ? t : count - 1;
+    double a = A[u], b = B[u], c = C[u], d = D[u], l = lo[u], h = hi[u];
+    const bool ok = quartic_ok(a, b, c, d, l, h);
+    if (!ok) a = b = d = l = h = 0.0, c = 1.0;
+    const double r = quartic_min64_seeded(a, b, c, d, l, h, mode);
+    if (in) x[t] = ok ? r : NAN;
+    const int nbad = in && !ok;
+    report_bad(nbad, bad);
 }
 
-__global__ void __launch_bounds__(256) quartic_many_f32(const float *A, const float *B, const float *C,
+// A pair with A = 0 or an invalid element, out of line.
+__device__ __noinline__ float2 quartic_pair_rest(float2 a, float2 b, float2 c, float2 d, float2 l, float2 h, int mode,
+                                                 int *nbad)
+{
+    unsigned esc = 0;
+    const bool okx = quartic_ok(a.x, b.x, c.x, d.x, l.x, h.x), oky = quartic_ok(a.y, b.y, c.y, d.y, l.y, h.y);
+    if (okx && oky) return quartic_min32_lanes(a, b, c, d, l, h, mode, &esc);
+    *nbad += (okx ? 0 : 1) + (oky ? 0 : 1);
+    return make_float2(okx ? quartic_min32(a.x, b.x, c.x, d.x, l.x, h.x, mode, esc) : NAN,
+                       oky ? quartic_min32(a.y, b.y, c.y, d.y, l.y, h.y, mode, esc) : NAN);
+}
+
+constexpr int kThreads32 = 128;
+__global__ void __launch_bounds__(kThreads32, 8) quartic_many_f32(const float *A, const float *B, const float *C,
                                                         const float *D, const float *lo, const float *hi,
                                                         int64_t count, int mode, float *x, int *bad)
 {
     const int64_t pairs = count / 2;
     unsigned esc = 0;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < pairs;
-         t += (int64_t)gridDim.x * blockDim.x) {
+    int nbad = 0;
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t < pairs) {
         const float2 a = ((const float2 *)A)[t], b = ((const float2 *)B)[t], c = ((const float2 *)C)[t],
                      d = ((const float2 *)D)[t], l = ((const float2 *)lo)[t], h = ((const float2 *)hi)[t];
-        const bool okx = quartic_ok(a.x, b.x, c.x, d.x, l.x, h.x), oky = quartic_ok(a.y, b.y, c.y, d.y, l.y, h.y);
+        // finite coefficients (their magnitudes' sum is), A > 0, lo <= hi; anything else is looked at lane by lane
+        const float2 m = add2(add2(abs2(a), abs2(b)), add2(abs2(c), abs2(d)));
         float2 r;
-        if (okx && oky) {
-            r = quartic_min32x2(a, b, c, d, l, h, mode, esc);
-        } else {
-            r.x = okx ? quartic_min32(a.x, b.x, c.x, d.x, l.x, h.x, mode, esc) : NAN;
-            r.y = oky ? quartic_min32(a.y, b.y, c.y, d.y, l.y, h.y, mode, esc) : NAN;
-            atomicAdd(bad, (okx ? 0 : 1) + (oky ? 0 : 1));
-        }
+        if (m.x < INFINITY && m.y < INFINITY && a.x > 0.0f && a.y > 0.0f && l.x <= h.x && l.y <= h.y)
+            r = quartic_min32x2_wells(a, b, c, d, l, h, mode, esc);
+        else
+            r = quartic_pair_rest(a, b, c, d, l, h, mode, &nbad);
         ((float2 *)x)[t] = r;
     }
     if (count % 2 == 1 && blockIdx.x == 0 && threadIdx.x == 0) {
-        const int64_t t = count - 1;
+        const int64_t t = count - 1; // the odd element
         if (quartic_ok(A[t], B[t], C[t], D[t], lo[t], hi[t])) {
             x[t] = quartic_min32(A[t], B[t], C[t], D[t], lo[t], hi[t], mode, esc);
         } else {
             x[t] = NAN;
-            atomicAdd(bad, 1);
+            ++nbad;
         }
     }
+    report_bad(nbad, bad);
 }
 
-int quartic_grid(int64_t work)
-{
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t want = (work + 255) / 256;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)std::max(nsm, 1) * 8));
-}
+// The calls' counters: words of one pinned, device-mapped host page, taken
+// by a call and given back when it returns (any thread, stream or device).
+// With every word taken, a call waits for none and allocates a page of its own.
+class BadWords {
+    static constexpr int kWords = 64, kStride = 32; // ints: one word per 128 bytes
+    std::mutex mu_;
+    int *page_ = nullptr;
+    uint64_t taken_ = 0;
+
+public:
+    struct Word {
+        int *p = nullptr;
+        int slot = -1; // -1: a page of its own
+    };
+    cudaError_t take(Word &w)
+    {
+        std::lock_guard<std::mutex> lk(mu_);
+        if (page_) { // gone if the device was reset since
+            cudaPointerAttributes at{};
+            if (cudaPointerGetAttributes(&at, page_) != cudaSuccess || at.type != cudaMemoryTypeHost) {
+                cudaGetLastError();
+                page_ = nullptr;
+                taken_ = 0;
+            }
+        }
+        if (!page_) {
+            const cudaError_t e = cudaHostAlloc((void **)&page_, sizeof(int) * kWords * kStride,
+                                                cudaHostAllocMapped | cudaHostAllocPortable);
+            if (e != cudaSuccess) return page_ = nullptr, e;
+        }
+        for (int t = 0; t < kWords; ++t)
+            if (!(taken_ >> t & 1)) {
+                taken_ |= 1ull << t;
+                w = {page_ + t * kStride, t};
+                *w.p = 0;
+                return cudaSuccess;
+            }
+        const cudaError_t e = cudaHostAlloc((void **)&w.p, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable);
+        if (e == cudaSuccess) *w.p = 0;
+        return e;
+    }
+    void give(Word &w)
+    {
+        if (!w.p) return;
+        if (w.slot < 0) {
+            cudaFreeHost(w.p);
+        } else {
+            std::lock_guard<std::mutex> lk(mu_);
+            taken_ &= ~(1ull << w.slot);
+        }
+        w.p = nullptr;
+    }
+};
+BadWords g_bad_words;
 
 template <class T>
 admm_status quartic_min_impl(const T *A, const T *B, const T *C, const T *D, const T *lo, const T *hi, int64_t count,
@@ -111,9 +190,10 @@ admm_status quartic_min_impl(const T *A, const T *B, const T *C, const T *D, con
     cudaStream_t st = (cudaStream_t)stream;
     const size_t bytes = sizeof(T) * (size_t)count;
     T *d[7] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    BadWords::Word bad;
     int *dbad = nullptr;
-    cudaError_t e = cudaMallocAsync(&dbad, sizeof(int), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dbad, 0, sizeof(int), st);
+    cudaError_t e = g_bad_words.take(bad);
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&dbad, bad.p, 0);
     const T *src[6] = {A, B, C, D, lo, hi};
     if (!on_device)
         for (int t = 0; t < 7 && e == cudaSuccess; ++t) {
@@ -125,21 +205,20 @@ admm_status quartic_min_impl(const T *A, const T *B, const T *C, const T *D, con
         for (int t = 0; t < 6; ++t) a[t] = on_device ? src[t] : d[t];
         T *xo = on_device ? x : d[6];
         if constexpr (sizeof(T) == 8)
-            quartic_many_f64<<<quartic_grid(count), 256, 0, st>>>(a[0], a[1], a[2], a[3], a[4], a[5], count,
+            quartic_many_f64<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(a[0], a[1], a[2], a[3], a[4], a[5], count,
                                                                   xmin_mode, xo, dbad);
         else
-            quartic_many_f32<<<quartic_grid(count / 2 + 1), 256, 0, st>>>(a[0], a[1], a[2], a[3], a[4], a[5],
+            quartic_many_f32<<<(unsigned)((count / 2 + kThreads32) / kThreads32), kThreads32, 0, st>>>(a[0], a[1], a[2], a[3], a[4], a[5],
                                                                           count, xmin_mode, xo, dbad);
         e = cudaGetLastError();
         if (e == cudaSuccess && !on_device) e = cudaMemcpyAsync(x, d[6], bytes, cudaMemcpyDeviceToHost, st);
     }
-    int hbad = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&hbad, dbad, sizeof(int), cudaMemcpyDeviceToHost, st);
     for (T *p : d)
         if (p) cudaFreeAsync(p, st);
-    if (dbad) cudaFreeAsync(dbad, st);
     const cudaError_t es = cudaStreamSynchronize(st);
     if (e == cudaSuccess) e = es;
+    const int hbad = e == cudaSuccess ? *(volatile int *)bad.p : 0;
+    g_bad_words.give(bad);
     if (e != cudaSuccess) {
         set_last_error(cudaGetErrorString(e));
         return e == cudaErrorMemoryAllocation ? ADMM_ENOMEM : ADMM_ECUDA;
