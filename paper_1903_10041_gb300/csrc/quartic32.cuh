@@ -26,15 +26,35 @@
 
 namespace admm_impl {
 
-// Fast FP32 primitives for the closed forms.  Their few-ulp errors are
-// removed by the Newton step that follows (the root it converges to depends
-// only on the coefficients), and the discriminant bound below allows for a
-// reciprocal that is off by 2 ulp.
-__device__ __forceinline__ float rcp_fast(float v) { return __fdividef(1.0f, v); }
-__device__ __forceinline__ float rsqrt_fast(float v) { return rsqrtf(v); }
-__device__ __forceinline__ float sqrt_fast(float v) { return v > 0.0f ? v * rsqrtf(v) : 0.0f; }
+// Fast FP32 primitives for the closed forms: single special-function
+// instructions that take denormals as zero (the forms that do not scale
+// operand and result around each, three to four instructions more).  Their
+// few-ulp errors are removed by the Newton step that follows (the root it
+// converges to depends only on the coefficients), and the discriminant bound
+// below allows for a reciprocal that is off by 2 ulp.  A denormal operand
+// gives an infinity or a zero, and with it a non-finite root or an
+// uncertified discriminant, which the callers send to FP64.
+__device__ __forceinline__ float rcp_fast(float v)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float rsqrt_fast(float v)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float sqrt_fast(float v) { return v > 0.0f ? v * rsqrt_fast(v) : 0.0f; }
 // |v|^(1/3) for v != 0
-__device__ __forceinline__ float cbrt_abs(float v) { return exp2f(__log2f(fabsf(v)) * (1.0f / 3.0f)); }
+__device__ __forceinline__ float cbrt_abs(float v)
+{
+    float l, r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(fabsf(v)));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(l * (1.0f / 3.0f)));
+    return r;
+}
 __device__ __forceinline__ float cbrt_fast(float v) { return copysignf(v != 0.0f ? cbrt_abs(v) : 0.0f, v); }
 
 // The FP64 closed form, out of line: taken only when FP32 overflows.
@@ -575,7 +595,7 @@ __device__ __forceinline__ float2 quartic_min32x2(float2 A, float2 B, float2 C, 
 // quartic benchmark, where a third are double wells and nearly every warp holds
 // both branches): both lanes' Cardano root and both lanes' trig roots are found
 // packed, and each lane keeps what its branch needs, instead of one lane after
-// the other through the scalar code (725 -> 347 warp instructions per 64
+// the other through the scalar code (725 -> 284 warp instructions per 64
 // quartics).  The decisions are those of quartic_min32: the branch outside
 // its error bound, the lower minimum where |br| of F(u) - F(v) = (u - v) br
 // exceeds 2e-5 of the sum of its terms' magnitudes (FP32 errs by a few 1e-7
