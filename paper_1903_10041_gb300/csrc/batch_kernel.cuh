@@ -33,6 +33,8 @@
 #pragma once
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "batch.h"
 #include "common.cuh"
 #include "mixed_elem.cuh"
@@ -227,43 +229,52 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
                 }
             }
             double *rec = recs + (size_t)(j + gw) * m * 4;
-            if constexpr (STG && ROLL) {
-                // one rolling stage per warp, each slot group refilled for round r + 1 as round r reads it
-                float2 *stw = stage + (size_t)wl * stage_region_slots<M>() * 32 + lane;
+            // PLAIN: not a check iteration, not cold, no pending mu divisor (nine iterations in
+            // ten), with those branches and their registers compiled out of the loop (not for M = 8,
+            // where two copies spill more than the branches cost)
+            auto columns = [&](auto plain) {
+                constexpr bool PLAIN = decltype(plain)::value;
+                const bool chk = !PLAIN && check, cld = !PLAIN && cold;
+                const float mud = PLAIN ? 1.0f : mu_div;
                 int v = v0 + lane;
-                roll_prologue<M>(ea, j, v * VW, v < v1, stw);
-                for (; v < v1; v += 32) {
-                    const int kn = v + 32 < v1 ? (v + 32) * VW : -1;
-                    vec32<M, VW, false, STAGE_ROLL>(ea, uoff, x1nu, j, v * VW, check, cold, mu_div, rho1, rho3,
-                                                    rho4, iq, ghi, glo, fmx, fmn, fcr, fcs, esc, rec, stw, kn);
-                }
-                cp_async_wait0();
-            } else if constexpr (STG) {
-                // two stages per warp; round r of the piece reads stage r & 1
-                // while the copies of round r + 1 fill the other
-                float2 *stw = stage + (size_t)wl * stage_region_slots<M>() * 32 + lane;
-                int v = v0 + lane;
-                if (v < v1) stage_vec32<M>(ea, j, v * VW, stw);
-                cp_async_commit();
-                for (int r = 0; v < v1; v += 32, ++r) {
-                    float2 *cur = stw + (r & 1) * stage_slots<M>() * 32;
-                    if (v + 32 < v1) {
-                        stage_vec32<M>(ea, j, (v + 32) * VW, stw + ((r + 1) & 1) * stage_slots<M>() * 32);
-                        prefetch_mutable<M>(ea, j, (v + 32) * VW);
+                if constexpr (STG && ROLL) {
+                    // one rolling stage per warp, each slot group refilled for round r + 1 as round r reads it
+                    float2 *stw = stage + (size_t)wl * stage_region_slots<M>() * 32 + lane;
+                    roll_prologue<M>(ea, j, v * VW, v < v1, stw);
+                    for (; v < v1; v += 32) {
+                        const int kn = v + 32 < v1 ? (v + 32) * VW : -1;
+                        vec32<M, VW, false, STAGE_ROLL>(ea, uoff, x1nu, j, v * VW, chk, cld, mud, rho1, rho3,
+                                                        rho4, iq, ghi, glo, fmx, fmn, fcr, fcs, esc, rec, stw, kn);
                     }
+                    cp_async_wait0();
+                } else if constexpr (STG) {
+                    // two stages per warp; round r of the piece reads stage r & 1
+                    // while the copies of round r + 1 fill the other
+                    float2 *stw = stage + (size_t)wl * stage_region_slots<M>() * 32 + lane;
+                    if (v < v1) stage_vec32<M>(ea, j, v * VW, stw);
                     cp_async_commit();
-                    cp_async_wait1(); // this round's copies have landed
-                    vec32<M, VW, false, STAGE_DOUBLE>(ea, uoff, x1nu, j, v * VW, check, cold, mu_div, rho1, rho3, rho4,
-                                              iq, ghi, glo, fmx, fmn, fcr, fcs, esc, rec, cur);
+                    for (int r = 0; v < v1; v += 32, ++r) {
+                        float2 *cur = stw + (r & 1) * stage_slots<M>() * 32;
+                        if (v + 32 < v1) {
+                            stage_vec32<M>(ea, j, (v + 32) * VW, stw + ((r + 1) & 1) * stage_slots<M>() * 32);
+                            prefetch_mutable<M>(ea, j, (v + 32) * VW);
+                        }
+                        cp_async_commit();
+                        cp_async_wait1(); // this round's copies have landed
+                        vec32<M, VW, false, STAGE_DOUBLE>(ea, uoff, x1nu, j, v * VW, chk, cld, mud, rho1, rho3,
+                                                          rho4, iq, ghi, glo, fmx, fmn, fcr, fcs, esc, rec, cur);
+                    }
+                    cp_async_wait0();
+                } else {
+                    for (; v < v1; v += 32) {
+                        if (v + 32 < v1) prefetch_vec32<M>(ea, j, (v + 32) * VW, cld);
+                        vec32<M, VW, false>(ea, uoff, x1nu, j, v * VW, chk, cld, mud, rho1, rho3, rho4, iq, ghi,
+                                            glo, fmx, fmn, fcr, fcs, esc, rec);
+                    }
                 }
-                cp_async_wait0();
-            } else {
-                for (int v = v0 + lane; v < v1; v += 32) {
-                    if (v + 32 < v1) prefetch_vec32<M>(ea, j, (v + 32) * VW, cold);
-                    vec32<M, VW, false>(ea, uoff, x1nu, j, v * VW, check, cold, mu_div, rho1, rho3, rho4, iq, ghi,
-                                        glo, fmx, fmn, fcr, fcs, esc, rec);
-                }
-            }
+            };
+            if (M > 4 || check || cold || mu_div != 1.0f) columns(std::false_type{});
+            else columns(std::true_type{});
 #pragma unroll
             for (int i = 0; i < M; ++i)
                 if (i < m) {
