@@ -1,0 +1,59 @@
+"""Results of a batch in device buffers (one launch) against the same results in host buffers, and the
+zero start set on the device against a new batch's, at the smallest and ragged sizes."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from paper_1903_10041_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def capi():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1903_10041_gb300 import build
+    build.build()
+    from paper_1903_10041_gb300 import capi
+    return capi
+
+
+@pytest.mark.parametrize("shapes", [[(1, 1, 1)], [(2, 1, 3), (37, 3, 5), (64, 2, 1), (1029, 4, 7)],
+                                    [(50, 8, 2), (33, 2, 31)]])
+def test_device_results_equal_host_results(capi, shapes):
+    import torch
+    P = [W.random_problem(n, m, q, seed=100 + t) for t, (n, m, q) in enumerate(shapes)]
+    par = W.Params(rho2_over_n=True, precision="mixed", max_iter=30)
+    dp = ctypes.POINTER(ctypes.c_double)
+    with capi.Batch(P, par) as b:
+        b.solve()
+        host = b.wait(want_x=True)
+        x = [torch.full((m * q * n + 1,), 7.0, dtype=torch.float64, device="cuda") for n, m, q in shapes]
+        x1 = [torch.full((m + 1,), 7.0, dtype=torch.float64, device="cuda") for n, m, q in shapes]
+        res = (capi.admm_result * len(P))()
+        for t, r in enumerate(res):
+            r.x = ctypes.cast(ctypes.c_void_p(x[t].data_ptr()), dp)
+            if t % 2 == 0:  # x alone for every second instance
+                r.x1 = ctypes.cast(ctypes.c_void_p(x1[t].data_ptr()), dp)
+            r.on_device = 1
+        st = capi._lib.admm_batch_wait(b.h, None, res)
+        assert st in (capi.ADMM_OK, capi.ADMM_ENOTCONVERGED)
+        for t, (n, m, q) in enumerate(shapes):
+            xt, x1t = x[t].cpu().numpy(), x1[t].cpu().numpy()
+            assert np.array_equal(xt[:-1].reshape(m, q, n), host[t]["x"]) and xt[-1] == 7.0
+            assert np.array_equal(x1t[:-1], host[t]["x1"]) if t % 2 == 0 else np.all(x1t == 7.0)
+            assert x1t[-1] == 7.0
+        # the zero start set on the device gives a new batch's state and solve
+        b.reset()
+        with capi.Batch(P, par) as fresh:
+            for t in range(len(P)):
+                s0, s1 = b.state(t), fresh.state(t)
+                for k in s0:
+                    assert np.array_equal(s0[k], s1[k]), k
+        b.solve()
+        again = b.wait(want_x=True)
+        for t in range(len(P)):
+            assert np.array_equal(again[t]["x"], host[t]["x"]) and again[t]["iters"] == host[t]["iters"]
