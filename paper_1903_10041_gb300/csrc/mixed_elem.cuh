@@ -351,8 +351,8 @@ __device__ __forceinline__ void vec32(const EA &a, const float *uoff, const floa
             const float2 g0 = cold ? ldg2(a.g0 + e) : splat2(0.0f);
             const int pr = i * q + j;
             const float2 x0 = xt[i];
-            const float2 gq_old = mul2(fma2(b2, x0, b1), x0);
-            const float2 u = cold ? neg2(g0) : add2(gq_old, splat2(uoff[pr]));
+            const float2 gx = fma2(b2, x0, b1);
+            const float2 u = cold ? neg2(g0) : fma2(gx, x0, splat2(uoff[pr])); // g(x~) + zeta + lambda
             const float2 others = sub2(xsum, x0); // sum over l != i (x_i is still x0 here)
             const float2 phi = add2(add2(sub2(st, others), yv), mu);
             const float2 hb2 = mul2(h1, b2); // (rho_1 / 2) b2; B = (rho_1 b2) b1 = hb2 (2 b1) exactly
@@ -362,8 +362,8 @@ __device__ __forceinline__ void vec32(const EA &a, const float *uoff, const floa
             float2 C = fma2(a2, iq2, fma2(h1, t, h3));
             float2 D = fma2(a1, iq2, fma2(mul2(nr1, b1), u, mul2(nr3, phi)));
             if (k0 == 0) {
-                C.x += 0.5f * rho4;
-                D.x -= rho4 * x1nu[pr];
+                C.x = fmaf(0.5f, rho4, C.x);
+                D.x = fmaf(-rho4, x1nu[pr], D.x); // the same rounding in every kernel that inlines this
             }
             float2 xn;
             if constexpr (C64)
@@ -384,7 +384,7 @@ __device__ __forceinline__ void vec32(const EA &a, const float *uoff, const floa
             }
             ff2_acc(ghi[i], glo[i], ghh, gll);
             if (check) {
-                const float2 dk = cold ? add2(ghh, g0) : sub2(ghh, gq_old);
+                const float2 dk = cold ? add2(ghh, g0) : sub2(ghh, mul2(gx, x0));
                 dmx[i] = fmaxf(dmx[i], v1 ? fmaxf(dk.x, dk.y) : dk.x);
                 dmn[i] = fminf(dmn[i], v1 ? fminf(dk.x, dk.y) : dk.x);
             }

@@ -150,15 +150,15 @@ __device__ __forceinline__ float quartic_min32(float A, float B, float C, float 
     const float c = __fmul_rn(__fmul_rn(0.5f, C), inv);
     const float d = __fmul_rn(__fmul_rn(0.25f, D), inv);
     const float b3 = __fmul_rn(b, 1.0f / 3.0f);
-    const float b3s = __fmul_rn(b3, b3), b3c = __fmul_rn(b3s, b3);
+    const float b3s = __fmul_rn(b3, b3);
     const float Q = __fmaf_rn(c, 1.0f / 3.0f, -b3s);
-    const float bhc = __fmul_rn(b3, __fmul_rn(0.5f, c));
-    const float R = __fsub_rn(__fsub_rn(bhc, b3c), __fmul_rn(0.5f, d));
+    const float hc = __fmul_rn(0.5f, c), hd = __fmul_rn(0.5f, d);
+    const float R = __fmaf_rn(b3, __fsub_rn(hc, b3s), -hd);
     const float Qs = __fmul_rn(Q, Q);
-    const float Dl = __fadd_rn(__fmul_rn(Qs, Q), __fmul_rn(R, R));
+    const float Dl = __fmaf_rn(Qs, Q, __fmul_rn(R, R));
     // magnitudes entering Q, R (including the rounding of b, c, d); |Q| <= mQ and |R| <= mR
     const float mQ = __fmaf_rn(fabsf(c), 1.0f / 3.0f, b3s);
-    const float mR = __fmaf_rn(0.5f, fabsf(d), __fadd_rn(fabsf(bhc), fabsf(b3c)));
+    const float mR = __fmaf_rn(fabsf(b3), __fadd_rn(b3s, fabsf(hc)), fabsf(hd));
     // |fl(Delta) - Delta| <= u (78 Q^2 mQ + 12 |Q|^3 + 88 |R| mR + 4 R^2) with u = 2^-24
     // (a factor 2 over the first-order propagation of the roundings above,
     // with a reciprocal of A off by up to 2 ulp).  As |Q|^3 <= Q^2 mQ and
@@ -177,8 +177,8 @@ __device__ __forceinline__ float quartic_min32(float A, float B, float C, float 
         // Delta > 0 here (certified, or FP64 said so): as in the packed path
         const float sq = Dl > 0.0f ? __fmul_rn(Dl, rsqrt_fast(Dl)) : 0.0f;
         const float S = cbrt_fast(__fadd_rn(R, R >= 0.0f ? sq : -sq));
-        const float T = S != 0.0f ? __fmul_rn(-Q, rcp_fast(S)) : 0.0f;
-        const float x = newton_polish32(A, B, C, D, __fsub_rn(__fadd_rn(S, T), b3));
+        const float ST = S != 0.0f ? __fmaf_rn(-Q, rcp_fast(S), S) : 0.0f; // S + T
+        const float x = newton_polish32(A, B, C, D, __fsub_rn(ST, b3));
         if (!isfinite(x)) return quartic_min_fallback64(A, B, C, D, lo, hi, paper_mode);
         return clampf(x, lo, hi);
     }
@@ -513,12 +513,37 @@ __device__ __forceinline__ double elem_min64_linear(double C, double Dh, double 
 // lane by lane by quartic_min32, so each lane gets the branch Algorithm 1
 // gives it.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// Written as PTX, each with its own rounding: the compiler fuses the builtins'
+// products into later sums where a product has one use, which made the bits
+// depend on what else a copy of the code needed the product for.
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    float2 r;
+    asm("{.reg .b64 p, q, s; mov.b64 p, {%2, %3}; mov.b64 q, {%4, %5}; add.rn.f32x2 s, p, q; mov.b64 {%0, %1}, s;}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b)
+{
+    float2 r;
+    asm("{.reg .b64 p, q, s; mov.b64 p, {%2, %3}; mov.b64 q, {%4, %5}; mul.rn.f32x2 s, p, q; mov.b64 {%0, %1}, s;}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    float2 r;
+    asm("{.reg .b64 p, q, s, t; mov.b64 p, {%2, %3}; mov.b64 q, {%4, %5}; mov.b64 t, {%6, %7};"
+        " fma.rn.f32x2 s, p, q, t; mov.b64 {%0, %1}, s;}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return r;
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, make_float2(-1.0f, -1.0f), a); }
 __device__ __forceinline__ float2 splat2(float v) { return make_float2(v, v); }
-__device__ __forceinline__ float2 neg2(float2 a) { return __fmul2_rn(a, make_float2(-1.0f, -1.0f)); }
+__device__ __forceinline__ float2 neg2(float2 a) { return mul2(a, make_float2(-1.0f, -1.0f)); }
 __device__ __forceinline__ float2 abs2(float2 a) { return make_float2(fabsf(a.x), fabsf(a.y)); }
 
 // Newton step of newton_polish32 on both lanes.
@@ -556,17 +581,15 @@ __device__ __forceinline__ float2 quartic_min32x2(float2 A, float2 B, float2 C, 
         const float2 c = mul2(mul2(splat2(0.5f), C), inv);
         const float2 d = mul2(mul2(splat2(0.25f), D), inv);
         const float2 b3 = mul2(b, splat2(1.0f / 3.0f));
-        const float2 b3s = mul2(b3, b3), b3c = mul2(b3s, b3);
-        const float2 Q = fma2(c, splat2(1.0f / 3.0f), neg2(b3s));
-        const float2 hc = mul2(splat2(0.5f), c);
-        const float2 bhc = mul2(b3, hc);
-        const float2 R = sub2(sub2(bhc, b3c), mul2(splat2(0.5f), d));
-        const float2 Qs = mul2(Q, Q);
-        const float2 Q3 = mul2(Qs, Q), R2 = mul2(R, R);
-        const float2 Dl = add2(Q3, R2);
+        const float2 b3s = mul2(b3, b3);
+        const float2 nQ = fma2(c, splat2(-1.0f / 3.0f), b3s); // -Q
+        const float2 hc = mul2(splat2(0.5f), c), nhd = mul2(splat2(-0.5f), d);
+        const float2 R = fma2(b3, sub2(hc, b3s), nhd);
+        const float2 Qs = mul2(nQ, nQ);
+        const float2 Dl = fma2(neg2(Qs), nQ, mul2(R, R));
         // the forward error bound of quartic_min32, on both lanes
         const float2 mQ = fma2(abs2(c), splat2(1.0f / 3.0f), b3s);
-        const float2 mR = fma2(splat2(0.5f), abs2(d), add2(abs2(bhc), abs2(b3c)));
+        const float2 mR = fma2(abs2(b3), add2(b3s, abs2(hc)), abs2(nhd));
         const float2 bound = mul2(splat2(7.68e-6f), fma2(Qs, mQ, mul2(abs2(R), mR)));
         if (Dl.x > bound.x && Dl.y > bound.y) { // Cardano on both lanes
             // here Delta > bound >= 0, so sqrt(Delta) > 0, |R +- sqrt(Delta)| > 0 and S != 0: the
@@ -576,8 +599,7 @@ __device__ __forceinline__ float2 quartic_min32x2(float2 A, float2 B, float2 C, 
             const float2 v = add2(R, make_float2(R.x >= 0.0f ? sq.x : -sq.x, R.y >= 0.0f ? sq.y : -sq.y));
             const float2 S = make_float2(copysignf(cbrt_abs(v.x), v.x), copysignf(cbrt_abs(v.y), v.y));
             const float2 rS = make_float2(rcp_fast(S.x), rcp_fast(S.y));
-            const float2 T = mul2(neg2(Q), rS);
-            const float2 x = newton_polish32x2(A, B, C, D, sub2(add2(S, T), b3));
+            const float2 x = newton_polish32x2(A, B, C, D, sub2(fma2(nQ, rS, S), b3)); // S + T - b/3
             if (isfinite(x.x) && isfinite(x.y))
                 return make_float2(clampf(x.x, lo.x, hi.x), clampf(x.y, lo.y, hi.y));
         }
@@ -628,12 +650,12 @@ __device__ __forceinline__ float2 quartic_min32x2_wells(float2 A, float2 B, floa
     const float2 b3 = mul2(b, splat2(1.0f / 3.0f));
     const float2 b3s = mul2(b3, b3);
     const float2 nQ = fma2(c, splat2(-1.0f / 3.0f), b3s); // -Q
-    const float2 hc = mul2(splat2(0.5f), c), hd = mul2(splat2(0.5f), d);
-    const float2 R = sub2(sub2(mul2(b3, hc), mul2(b3s, b3)), hd);
+    const float2 hc = mul2(splat2(0.5f), c), nhd = mul2(splat2(-0.5f), d);
+    const float2 R = fma2(b3, sub2(hc, b3s), nhd);
     const float2 Qs = mul2(nQ, nQ);
-    const float2 Dl = sub2(mul2(R, R), mul2(Qs, nQ));
+    const float2 Dl = fma2(neg2(Qs), nQ, mul2(R, R));
     // the forward error bound of quartic_min32, on both lanes
-    const float2 ahc = abs2(hc), ahd = abs2(hd);
+    const float2 ahc = abs2(hc), ahd = abs2(nhd), nb3 = neg2(b3);
     const float2 mQ = fma2(ahc, splat2(2.0f / 3.0f), b3s);
     const float2 mR = fma2(abs2(b3), add2(b3s, ahc), ahd);
     const float2 bound = mul2(splat2(7.68e-6f), fma2(Qs, mQ, mul2(abs2(R), mR)));
@@ -647,14 +669,14 @@ __device__ __forceinline__ float2 quartic_min32x2_wells(float2 A, float2 B, floa
     {
         const float2 w = add2(R, make_float2(R.x >= 0.0f ? sq.x : -sq.x, R.y >= 0.0f ? sq.y : -sq.y));
         const float2 S = make_float2(copysignf(cbrt_abs(w.x), w.x), copysignf(cbrt_abs(w.y), w.y));
-        u = sub2(fma2(nQ, make_float2(rcp_fast(S.x), rcp_fast(S.y)), S), b3);
+        u = add2(fma2(nQ, make_float2(rcp_fast(S.x), rcp_fast(S.y)), S), nb3);
     }
     const bool any_trig = __any_sync(__activemask(), tx || ty);
     if (any_trig) {
         const float2 arg = max2(min2(mul2(R, mul2(rs, mul2(rs, rs))), splat2(1.0f)), splat2(-1.0f));
         const float2 sq2 = add2(sq, sq);
-        v = sub2(mul2(sq2, cos_third2(arg)), b3);
-        u = sel2(tx, ty, neg2(fma2(sq2, cos_third2(neg2(arg)), b3)), u);
+        v = fma2(sq2, cos_third2(arg), nb3);
+        u = sel2(tx, ty, fma2(neg2(sq2), cos_third2(neg2(arg)), nb3), u);
         v = newton_polish32x2(A, B, C, D, v);
         v = sel2(tx, ty, v, u);
     }
@@ -665,12 +687,11 @@ __device__ __forceinline__ float2 quartic_min32x2_wells(float2 A, float2 B, floa
     if (any_trig) {
         const float2 vc = max2(min2(v, hi), lo);
         const float2 p = paper_mode ? u : x, r = paper_mode ? v : vc;
-        const float2 s = add2(p, r), pp = mul2(p, p), rr = mul2(r, r), pr = mul2(p, r);
-        const float2 q2 = add2(pp, rr), q3 = add2(q2, pr);
-        const float2 as = add2(abs2(p), abs2(r)), b3q = mul2(b3, q3), cs = mul2(hc, s);
+        const float2 s = add2(p, r), q2 = fma2(p, p, mul2(r, r)), q3 = fma2(p, r, q2);
+        const float2 as = add2(abs2(p), abs2(r)), b3q = mul2(b3, q3);
         // br = (u^3 + u^2 v + u v^2 + v^3) / 4 + (b/3) (u^2 + u v + v^2) + (c/2) (u + v) + d
         const float2 q4 = mul2(splat2(0.25f), q2);
-        const float2 br = add2(add2(fma2(q4, s, b3q), cs), d);
+        const float2 br = add2(fma2(q4, s, b3q), fma2(hc, s, d));
         const float2 mb = add2(fma2(q4, as, abs2(b3q)), fma2(ahc, as, add2(ahd, ahd)));
         const float2 lim = mul2(splat2(2.0e-5f), mb);
         const bool nx = tx && p.x != r.x, ny = ty && p.y != r.y; // u < v: the larger root where br < 0

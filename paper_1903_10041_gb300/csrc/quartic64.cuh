@@ -44,11 +44,12 @@ __device__ __forceinline__ float rcp_approx_f32(float v)
 // FP64 element update does its comparisons and conversions on the integer
 // pipes.
 
-// (float)v, rounded to nearest (halves away from zero); magnitudes below the
-// FP32 normal range give a signed zero, above it (and infinities, NaN) an infinity.
+// (float)v, rounded to nearest even; magnitudes below the FP32 normal range
+// give a signed zero, above it (and infinities, NaN) an infinity.
 __device__ __forceinline__ float f64_to_f32_int(double v)
 {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v) + 0x10000000ull;
+    const unsigned long long w = (unsigned long long)__double_as_longlong(v);
+    const unsigned long long b = w + 0x0fffffffull + ((unsigned)w >> 29 & 1u);
     const unsigned hi = (unsigned)(b >> 32), ah = hi & 0x7fffffffu;
     const unsigned f = ((unsigned)(b >> 29) - (896u << 23)) & 0x7fffffffu;
     const unsigned r = ah < (897u << 20) ? 0u : (ah >= (1151u << 20) ? 0x7f800000u : f);

@@ -57,3 +57,47 @@ def test_device_results_equal_host_results(capi, shapes):
         again = b.wait(want_x=True)
         for t in range(len(P)):
             assert np.array_equal(again[t]["x"], host[t]["x"]) and again[t]["iters"] == host[t]["iters"]
+
+
+@pytest.mark.parametrize("cfg", [(16, 0, 0, 1, 0), (8, 0, 4096, 1, 0), (8, 0, 0, 2, 2048)])
+def test_a_batch_resumed_anywhere_gives_the_same_bits(capi, cfg):
+    """A solve cut at any iteration (a check there, where the whole run has none) and continued from its
+    saved state takes the whole run's bits: check and plain iterations round alike, and the scalar state
+    read back gives the same FP32 offsets as the one kept on chip (ties among them: q = 2 means)."""
+    shapes = [(276, 4, 18), (139, 4, 6), (600, 2, 2), (77, 3, 2), (33, 1, 1)]
+    P = [W.random_problem(n, m, q, seed=300 + t) for t, (n, m, q) in enumerate(shapes)]
+
+    def run(iters, states=None):
+        par = W.Params(rho=(1.0, 1.0 / 600, 1.0, 1.0), precision="mixed", max_iter=iters)
+        with capi.Batch(P, par) as b:
+            b.set_config(*cfg)
+            for t, s in enumerate(states or []):
+                b.set_state(t, s)
+            b.solve()
+            b.wait()
+            return [b.state(t) for t in range(len(P))]
+
+    whole = run(47)
+    for cut in (1, 10, 23):
+        part = run(47 - cut, run(cut))
+        for t in range(len(P)):
+            for k in whole[t]:
+                assert np.array_equal(whole[t][k], part[t][k]), (cut, t, k)
+
+
+@pytest.mark.parametrize("precision,n,m,q", [("mixed", 600, 2, 2), ("mixed", 2003, 4, 6), ("mixed", 301, 6, 3),
+                                             ("fp64", 301, 3, 2)])
+def test_a_single_solve_resumed_anywhere_gives_the_same_bits(capi, precision, n, m, q):
+    P = W.random_problem(n, m, q, seed=77)
+
+    def run(iters, warm=None):
+        par = W.Params(rho=(1.0, 1.0 / n, 1.0, 1.0), precision=precision, max_iter=iters)
+        with capi.Solver(P, par) as s:
+            s.solve(warm=warm)
+            return s.state()
+
+    whole = run(47)
+    for cut in (1, 10, 23):
+        part = run(47 - cut, run(cut))
+        for k in whole:
+            assert np.array_equal(whole[k], part[k]), (cut, k)
