@@ -129,9 +129,9 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
     const int64_t npairs = (int64_t)q * nv;
     const int items = q + W - 1; // record slots: (row j, warp w) at j + w
 
-    // shared memory: scal | rec[2][items][m][4] | cmax[2][NWT][2] | part[24] | x0s[mq] | x1n | scr | uoff | x1nu
-    // part: [0], [1] end-of-solve sums; [2] kappa; [3] the adaptation factor of a check; [16..19] fpar;
-    // [20..23] ipar.  Thread 0 keeps these team-wide values current so that the other threads read them
+    // shared memory: scal | rec[2][items][m][4] | cmax[2][NWT][2] | part[24] | x0s[mq] | scr | uoff | x1nu | rows[q]
+    // part: [0], [1] end-of-solve sums; [2] kappa; [3] the adaptation factor of a check; [4] 1/q; [5] n;
+    // [16..19] fpar; [20..23] ipar.  Thread 0 keeps these team-wide values current so that the other threads read them
     // instead of each converting and dividing on the FP64 pipe.
     double *scal = smem;
     double *lam = scal, *zeta = scal + mq, *hh = scal + 2 * mq, *pp = scal + 3 * mq, *nu = scal + 4 * mq;
@@ -139,13 +139,13 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
     double *rec0 = smem + scal_size(m, q);
     double *cmax = rec0 + 2 * (size_t)items * m * 4;
     double *part = cmax + 4 * NWT;
-    float *fpar = (float *)(part + 16); // rho_1, rho_3, rho_4 and the pending mu divisor, in FP32
-    int *ipar = (int *)(part + 20);     // converged, penalties changed, cold start
+    float *fpar = (float *)(part + 16); // rho_1, rho_3, rho_4, the pending mu divisor and 1/q, in FP32
+    int *ipar = (int *)(part + 20);     // converged, penalties changed, cold start, log2 of the lanes per pair
     double *x0s = part + 24;
-    double *x1n = x0s + mq;
-    double *scr = x1n + kMaxM;
+    double *scr = x0s + mq;
     float *uoff = (float *)(scr + kWarpsMax * 8); // [mq] (float)(zeta + lambda)
     float *x1nu = uoff + mq;                      // [mq] (float)(x1 + nu)
+    int *rows = (int *)(x1nu + mq);               // [q] first warp whose range covers row j, how many << 16
 
     double *gscal = a.scal + I.off_scal;
     double *out = a.out + (size_t)id * kInfo;
@@ -159,14 +159,28 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
         x1nu[pr] = (float)(x1[pr / q] + nu[pr]);
     }
     if (tid == 0) {
-        part[2] = rho[1] / (rho[0] + (double)n * rho[1]); // kappa of step (b)
+        part[2] = rho[1] / fma((double)n, rho[1], rho[0]); // kappa of step (b)
         fpar[0] = (float)rho[0];
         fpar[1] = (float)rho[2];
         fpar[2] = (float)rho[3];
         fpar[3] = (float)flags[1];
         ipar[2] = flags[0] != 0.0;
     }
+    for (int j = tid; j < q; j += NTL) {
+        const int wf = (int)((int64_t)j * nv / chunk);
+        rows[j] = wf | ((int)(((int64_t)j * nv + nv - 1) / chunk) - wf + 1) << 16;
+    }
     const int it0 = (int)__ldcg(out);
+    if (tid == 0) {
+        part[4] = 1.0 / (double)q;
+        part[5] = (double)n;
+        fpar[4] = 1.0f / (float)q;
+        // lanes that share the records of one pair in the scalar steps (log2)
+        const int most = (int)((nv + chunk - 1) / chunk) + 1;
+        int g = 0;
+        while ((2 << g) <= most && g < 5 && (mq << (g + 1)) <= NTL) ++g;
+        ipar[3] = g;
+    }
     sync_local();
 
     // the arrays' bases and this instance's 32-bit offsets into them (the arrays hold < 2^32 elements)
@@ -192,14 +206,15 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
     }
     const int it_end = budget > 0 ? (int)min((int64_t)a.max_iter, (int64_t)it0 + budget) : a.max_iter;
 
+    int ncheck = a.check_every - it % a.check_every; // iterations up to the next check
     while (it < it_end) {
         ++it;
         const int par = it & 1;
-        const bool check = (it % a.check_every == 0) || (it == a.max_iter);
+        const bool check = --ncheck == 0 || it == a.max_iter;
+        if (ncheck == 0) ncheck = a.check_every;
         const bool cold = ipar[2] != 0;
         const float mu_div = fpar[3];
-        const float rho1 = fpar[0], rho3 = fpar[1], rho4 = fpar[2];
-        const float iq = 1.0f / (float)q;
+        const float rho1 = fpar[0], rho3 = fpar[1], rho4 = fpar[2], iq = fpar[4];
         // lane maxima and minima that only check iterations use: with the staged
         // (m <= 4) update they live in the thread's own shared-memory slots (11
         // floats apart, no bank conflicts) instead of registers across the loop
@@ -275,32 +290,37 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
             };
             if (M > 4 || check || cold || mu_div != 1.0f) columns(std::false_type{});
             else columns(std::true_type{});
+            {
+                // the piece's sums of all sources at once (warp_many), written by one lane per source
+                auto add = [](FF k, FF u, int o) {
+                    return ff_add(k, FF{__shfl_xor_sync(0xffffffffu, u.hi, o), __shfl_xor_sync(0xffffffffu, u.lo, o)});
+                };
+                FF g[M];
 #pragma unroll
-            for (int i = 0; i < M; ++i)
-                if (i < m) {
-                    FF v = lanes_sum(ghi[i], glo[i]);
-                    float hi = check ? fmx[i] : 0.0f, lo = check ? fmn[i] : 0.0f;
+                for (int i = 0; i < M; ++i) g[i] = lanes_sum(ghi[i], glo[i]);
+                const FF v = warp_many<M>(g, add);
+                const int i = slot_of<M>(lane);
+                const bool out_lane = lane % (32 / M) == 0 && i < m;
+                if (out_lane) rec[i * 4 + 0] = f32_to_f64_int(v.hi) + f32_to_f64_int(v.lo);
+                if (check) {
+                    auto mx = [](float k, float u, int o) { return fmaxf(k, __shfl_xor_sync(0xffffffffu, u, o)); };
+                    auto mn = [](float k, float u, int o) { return fminf(k, __shfl_xor_sync(0xffffffffu, u, o)); };
+                    float th[M], tl[M];
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        const FF u = {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
-                        v = ff_add(v, u);
-                        if (check) {
-                            hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-                            lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-                        }
-                    }
-                    if (lane == 0) {
-                        rec[i * 4 + 0] = (double)v.hi + (double)v.lo;
-                        rec[i * 4 + 1] = check ? (double)hi : 0.0;
-                        rec[i * 4 + 2] = check ? (double)lo : 0.0;
+                    for (int t = 0; t < M; ++t) th[t] = fmx[t], tl[t] = fmn[t];
+                    const float hi = warp_many<M>(th, mx), lo = warp_many<M>(tl, mn);
+                    if (out_lane) {
+                        rec[i * 4 + 1] = f32_to_f64_int(hi);
+                        rec[i * 4 + 2] = f32_to_f64_int(lo);
                     }
                 }
+            }
         }
         if (check) {
             const float wr = warp_max(fcr), ws = warp_max(fcs);
             if (lane == 0) {
-                cmax[(par * NWT + wl) * 2 + 0] = (double)wr;
-                cmax[(par * NWT + wl) * 2 + 1] = (double)ws;
+                cmax[(par * NWT + wl) * 2 + 0] = f32_to_f64_int(wr);
+                cmax[(par * NWT + wl) * 2 + 1] = f32_to_f64_int(ws);
             }
         }
         sync_team(); // every record of this iteration is complete and visible
@@ -309,109 +329,135 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
             fpar[3] = 1.0f;
         }
 
-        const double kappa = part[2];
-        double r2m = 0.0, r3m = 0.0, s1m = 0.0, s2m = 0.0;
-        for (int pr = tid; pr < mq; pr += NTL) {
-            const int i = pr / q, j = pr - i * q;
-            double Ssum = 0.0, dmx = -INFINITY, dmn = INFINITY, x0 = 0.0;
-            const int wf = (int)((int64_t)j * nv / chunk), wlst = (int)(((int64_t)j * nv + nv - 1) / chunk);
-            for (int w = wf; w <= wlst; ++w) { // the warps whose ranges cover row j, in order
-                const double *rb = recs;
-                if constexpr (KIND == TEAM_CLUSTER) rb = cg::this_cluster().map_shared_rank(recs, w / NWT);
-                const double *rr = rb + ((size_t)(j + w) * m + i) * 4;
-                Ssum += rr[0];
-                if (check) {
-                    dmx = fmax(dmx, rr[1]);
-                    dmn = fmin(dmn, rr[2]);
-                }
-                if (w == wf) x0 = (double)*(const float *)(rr + 3); // k = 0 lies in the first warp's piece
-            }
-            const double lm = lam[pr], zt = zeta[pr], h0 = hh[pr], p0 = pp[pr];
-            const double Wv = (Ssum + sumg0[pr]) - (double)n * lm;
-            const double lamn = kappa * ((h0 + p0) - Wv);
-            const double Z = Wv + (double)n * lamn;
-            const double cz = Z - p0;
-            const double hn = cz < cc[i] ? cz : cc[i];
-            const double pn = p0 + (hn - Z);
-            if (check) {
-                r2m = max_nonneg(r2m, fabs(lamn - lm));
-                r3m = max_nonneg(r3m, fabs(hn - Z));
-                const double dl = (lamn - lm) - zt;
-                s1m = max_nonneg(s1m, max_nonneg(fabs(dmx + dl), fabs(dmn + dl)));
-                s2m = max_nonneg(s2m, fabs(hn - h0));
-            }
-            lam[pr] = lamn;
-            zeta[pr] = lamn - lm;
-            hh[pr] = hn;
-            pp[pr] = pn;
-            x0s[pr] = x0;
-        }
-        sync_local();
-        for (int i = tid >> 5; i < m; i += NTL / 32) { // (c), mean over j: one warp per source
-            const int lane = tid & 31;
-            double sum = 0.0;
-            for (int j = lane; j < q; j += 32) sum += x0s[i * q + j] - nu[i * q + j];
-            sum = warp_sum(sum);
-            if (lane == 0) x1n[i] = sum / (double)q;
-        }
-        sync_local();
-        // (h), and the FP32 offsets of the next element phase (lambda, zeta final; x1 = x1n)
-        double r4m = 0.0;
-        for (int pr = tid; pr < mq; pr += NTL) {
-            const int i = pr / q;
-            const double x0 = x0s[pr], xn = x1n[i];
-            const double nun = nu[pr] + (xn - x0);
-            nu[pr] = nun;
-            uoff[pr] = (float)(zeta[pr] + lam[pr]);
-            x1nu[pr] = (float)(xn + nun);
-            if (check) r4m = max_nonneg(r4m, fabs(x0 - xn));
-        }
-        if (tid < m) x1[tid] = x1n[tid];
         if (tid == 0) {
             flags[0] = 0.0;
             ipar[2] = 0;
         }
+        // The scalar steps, two independent chains on different warps with one barrier after both:
+        // the mean over j of step (c) with (h), one warp per source from the last warp down, and
+        // steps (b), (d), (g), (i) per pair, G lanes sharing a pair's records.  Bound by latency (a
+        // chain of about 15 FP64 instructions of 64 cycles): comparisons, conversions and the
+        // records' row ranges (once per solve) stay off the FP64 pipe and out of the loop.  4096
+        // adaptive solves 767 -> 691 ms, a burst of 48 served solves (n <= 600) 129 -> 104 ms.
+        double r2m = 0.0, r3m = 0.0, r4m = 0.0, s1m = 0.0, s2m = 0.0;
+        for (int i = NWT - 1 - wl; i < m; i += NWT) {
+            double sum = 0.0;
+            for (int j = lane; j < q; j += 32) {
+                const int w = rows[j] & 0xffff; // k = 0 lies in the first warp's piece
+                const double *rb = recs;
+                if constexpr (KIND == TEAM_CLUSTER) rb = cg::this_cluster().map_shared_rank(recs, w / NWT);
+                const double x0 = f32_to_f64_int(*(const float *)(rb + ((size_t)(j + w) * m + i) * 4 + 3));
+                const double d = x0 - nu[i * q + j];
+                x0s[i * q + j] = x0;
+                sum = j == lane ? d : sum + d;
+            }
+            const double xn = __dmul_rn(warp_sum(sum), part[4]);         // (c), the mean over j; not fused into (h)
+            for (int j = lane; j < q; j += 32) {
+                const int pr = i * q + j;
+                const double d = xn - x0s[pr], nun = nu[pr] + d;      // (h)
+                nu[pr] = nun;
+                x1nu[pr] = f64_to_f32_int(xn + nun);
+                if (check) r4m = max_nonneg(r4m, fabs(d));
+            }
+            if (lane == 0) x1[i] = xn;
+        }
+        const double kappa = part[2], nd = part[5];
+        const int gsh = ipar[3], G = 1 << gsh;
+        for (int p0 = 0; p0 < mq; p0 += NTL >> gsh) {
+            if (p0 + ((tid & ~31) >> gsh) >= mq) break; // the whole warp is past the pairs
+            const int pq = p0 + (tid >> gsh), sub = tid & (G - 1);
+            const bool in = pq < mq;
+            const int pr = in ? pq : mq - 1;
+            const int i = pr / q, j = pr - i * q;
+            const int wf = rows[j] & 0xffff, nw = rows[j] >> 16;
+            const double g0s = sumg0[pr], ci = cc[i];
+            double S = 0.0, dmx = -INFINITY, dmn = INFINITY;
+            for (int t = sub; t < nw; t += G) { // the warps whose ranges cover row j, in order
+                const double *rb = recs;
+                if constexpr (KIND == TEAM_CLUSTER) rb = cg::this_cluster().map_shared_rank(recs, (wf + t) / NWT);
+                const double *rr = rb + ((size_t)(j + wf + t) * m + i) * 4;
+                S = t == sub ? rr[0] : S + rr[0];
+                if (check) {
+                    dmx = max_ord(dmx, rr[1]);
+                    dmn = min_ord(dmn, rr[2]);
+                }
+            }
+            for (int o = G >> 1; o > 0; o >>= 1) {
+                S += __shfl_xor_sync(0xffffffffu, S, o);
+                if (check) {
+                    dmx = max_ord(dmx, __shfl_xor_sync(0xffffffffu, dmx, o));
+                    dmn = min_ord(dmn, __shfl_xor_sync(0xffffffffu, dmn, o));
+                }
+            }
+            const double lm = lam[pr], zt = zeta[pr], h0 = hh[pr], pv = pp[pr];
+            const double Wv = fma(-nd, lm, S + g0s);                  // 1'(g(x) - lambda)
+            const double lamn = __dmul_rn(kappa, (h0 + pv) - Wv);     // (b) + (g); never fused into later sums,
+                                                                      // which a resumed solve forms from lamn
+            const double Z = fma(nd, lamn, Wv);                       // 1'z
+            const double hn = min_ord(Z - pv, ci);                    // (d)
+            const double e = hn - Z, zn = lamn - lm;
+            if (check && in) { // a lane past the pairs may see the last pair's new scalars
+                r2m = max_nonneg(r2m, fabs(zn));
+                r3m = max_nonneg(r3m, fabs(e));
+                const double dl = zn - zt;
+                s1m = max_nonneg(s1m, max_nonneg(fabs(dmx + dl), fabs(dmn + dl)));
+                s2m = max_nonneg(s2m, fabs(hn - h0));
+            }
+            __syncwarp(); // the lanes of a pair have read its scalars
+            if (in && sub == 0) {
+                lam[pr] = lamn;
+                zeta[pr] = zn;
+                hh[pr] = hn;
+                pp[pr] = pv + e;                                      // (i)
+                uoff[pr] = f64_to_f32_int(zn + lamn);
+            }
+        }
+        if (check) { // per-warp maxima of the residual terms
+            double v[8] = {r2m, r3m, r4m, s1m, s2m, 0.0, 0.0, 0.0};
+            auto mx = [](double k, double u, int o) { return max_nonneg(k, __shfl_xor_sync(0xffffffffu, u, o)); };
+            const double r = warp_many<8>(v, mx);
+            if ((lane & 3) == 0) scr[wl * 8 + (lane >> 2)] = r;
+        }
         sync_local();
         if (check) {
-            // maxima of the residual terms: per warp, then over the team's warps and (for a cluster)
-            // the CTAs' column maxima by thread 0, which takes the stop decision and the adaptation
-            // of Sec. IV-A and passes them on; every CTA of a cluster decides the same way
-            double v[5] = {r2m, r3m, r4m, s1m, s2m};
-#pragma unroll
-            for (int t = 0; t < 5; ++t) v[t] = warp_max_nonneg(v[t]);
-            if constexpr (KIND != TEAM_WARP) {
-                if (lane == 0)
-                    for (int t = 0; t < 5; ++t) scr[wl * 8 + t] = v[t];
-                sync_local();
-            }
-            if (tid == 0) {
-                double w[7] = {0.0, v[0], v[1], v[2], v[3], v[4], 0.0};
-                if constexpr (KIND != TEAM_WARP)
-                    for (int ww = 0; ww < NWT; ++ww)
-                        for (int t = 0; t < 5; ++t) w[1 + t] = max_nonneg(w[1 + t], scr[ww * 8 + t]);
-                for (int r = 0; r < CL; ++r) {
+            // over the team's warps and (for a cluster) the CTAs' column maxima by the first warp, whose
+            // lane 0 takes the stop decision and the adaptation of Sec. IV-A and passes them on; every
+            // CTA of a cluster decides the same way
+            if (wl == 0) {
+                double c0 = 0.0, c1 = 0.0, v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+                for (int t = lane; t < W; t += 32) {
                     const double *cb = cmax;
-                    if constexpr (KIND == TEAM_CLUSTER) cb = cg::this_cluster().map_shared_rank(cmax, r);
-                    for (int ww = 0; ww < NWT; ++ww) {
-                        w[0] = max_nonneg(w[0], cb[(par * NWT + ww) * 2 + 0]);
-                        w[6] = max_nonneg(w[6], cb[(par * NWT + ww) * 2 + 1]);
+                    if constexpr (KIND == TEAM_CLUSTER) cb = cg::this_cluster().map_shared_rank(cmax, t / NWT);
+                    c0 = max_nonneg(c0, cb[(par * NWT + t % NWT) * 2 + 0]);
+                    c1 = max_nonneg(c1, cb[(par * NWT + t % NWT) * 2 + 1]);
+                }
+                v[5] = c0;
+                v[6] = c1;
+                if (lane < NWT)
+#pragma unroll
+                    for (int t = 0; t < 5; ++t) v[t] = scr[lane * 8 + t];
+                auto mx = [](double k, double u, int o) { return max_nonneg(k, __shfl_xor_sync(0xffffffffu, u, o)); };
+                const double mine = warp_many<8>(v, mx); // value lane / 4
+                double w[7];
+#pragma unroll
+                for (int t = 0; t < 7; ++t) w[t] = __shfl_sync(0xffffffffu, mine, (t == 0 ? 5 : t == 6 ? 6 : t - 1) * 4);
+                if (lane == 0) {
+                    for (int t = 0; t < 7; ++t) res[t] = w[t];
+                    const double r = max_nonneg(max_nonneg(w[0], w[1]), max_nonneg(w[2], w[3]));
+                    const double sgm = max_nonneg(max_nonneg(rho[0] * w[4], rho[1] * w[5]), rho[2] * w[6]);
+                    r_last = r;
+                    s_last = sgm;
+                    const bool cv = r < a.r_tol && sgm < a.s_tol;
+                    double f = 1.0;
+                    if (!cv && a.adapt && it < a.max_iter && it >= a.adapt_start) { // Sec. IV-A, duals rescaled
+                        const double ratio = r / sgm, target = a.adapt_target;
+                        if (ratio > 1.2 * target) f = a.tau;
+                        else if (ratio < 0.8 * target) f = 1.0 / a.tau;
                     }
+                    ipar[0] = cv;
+                    ipar[1] = f != 1.0;
+                    part[3] = f;
                 }
-                for (int t = 0; t < 7; ++t) res[t] = w[t];
-                const double r = fmax(fmax(w[0], w[1]), fmax(w[2], w[3]));
-                const double sgm = fmax(fmax(rho[0] * w[4], rho[1] * w[5]), rho[2] * w[6]);
-                r_last = r;
-                s_last = sgm;
-                const bool cv = r < a.r_tol && sgm < a.s_tol;
-                double f = 1.0;
-                if (!cv && a.adapt && it < a.max_iter && it >= a.adapt_start) { // Sec. IV-A, duals rescaled
-                    const double ratio = r / sgm, target = a.adapt_target;
-                    if (ratio > 1.2 * target) f = a.tau;
-                    else if (ratio < 0.8 * target) f = 1.0 / a.tau;
-                }
-                ipar[0] = cv;
-                ipar[1] = f != 1.0;
-                part[3] = f;
             }
             sync_local();
             if (ipar[0]) {
@@ -430,7 +476,7 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
                 if (tid == 0) {
                     for (int t = 0; t < 4; ++t) rho[t] *= f;
                     flags[1] = f;
-                    part[2] = rho[1] / (rho[0] + (double)n * rho[1]);
+                    part[2] = rho[1] / fma((double)n, rho[1], rho[0]);
                     fpar[0] = (float)rho[0];
                     fpar[1] = (float)rho[2];
                     fpar[2] = (float)rho[3];

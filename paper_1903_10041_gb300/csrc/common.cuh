@@ -124,6 +124,36 @@ template <class T> __device__ __forceinline__ T warp_min(T v)
     return v;
 }
 
+// Warp sums (or maxima, minima) of M values per lane at once: while more than
+// one value is left, a step halves the values by keeping one half in the
+// lanes with the step's bit clear and the other in those with it set, so M
+// values take M - 1 + log2(32 / M) combinations instead of 5 M.  The total of
+// value slot_of<M>(lane) ends up in every lane of its group of 32 / M.
+template <int M> __device__ __forceinline__ int slot_of(int lane)
+{
+    return M == 2 ? lane >> 4 : (M == 4 ? lane >> 3 : lane >> 2);
+}
+template <int M, class T, class F> __device__ __forceinline__ T warp_many(T *v, F comb)
+{
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int c = M; c > 1; c >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int t = 0; t < M / 2; ++t)
+            if (t < c / 2) {
+                const T keep = up ? v[t + c / 2] : v[t], send = up ? v[t] : v[t + c / 2];
+                v[t] = comb(keep, send, o);
+            }
+        o >>= 1;
+    }
+    T r = v[0];
+#pragma unroll
+    for (int u = 16 / M; u > 0; u >>= 1) r = comb(r, r, u);
+    return r;
+}
+
 __device__ __forceinline__ double clampd(double v, double lo, double hi)
 {
     return v < lo ? lo : (v > hi ? hi : v);

@@ -110,36 +110,6 @@ __device__ __forceinline__ Sm carve(double *base, int m, int q)
     return s;
 }
 
-// Warp sums (or maxima, minima) of M values per lane at once: while more than
-// one value is left, a step halves the values by keeping one half in the
-// lanes with the step's bit clear and the other in those with it set, so M
-// values take M - 1 + log2(32 / M) combinations instead of 5 M.  The total of
-// value slot_of<M>(lane) ends up in every lane of its group of 32 / M.
-template <int M> __device__ __forceinline__ int slot_of(int lane)
-{
-    return M == 2 ? lane >> 4 : (M == 4 ? lane >> 3 : lane >> 2);
-}
-template <int M, class T, class F> __device__ __forceinline__ T warp_many(T *v, F comb)
-{
-    const int lane = threadIdx.x & 31;
-    int o = 16;
-#pragma unroll
-    for (int c = M; c > 1; c >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int t = 0; t < M / 2; ++t)
-            if (t < c / 2) {
-                const T keep = up ? v[t + c / 2] : v[t], send = up ? v[t] : v[t + c / 2];
-                v[t] = comb(keep, send, o);
-            }
-        o >>= 1;
-    }
-    T r = v[0];
-#pragma unroll
-    for (int u = 16 / M; u > 0; u >>= 1) r = comb(r, r, u);
-    return r;
-}
-
 // Per-iteration constants of the FP64 element update, the same in every thread.
 struct Iter64 {
     double rho3h, rho4h, hr1, iq, iqh; // rho_3/2, rho_4/2, rho_1/2, 1/q, 1/(2q)
@@ -473,7 +443,7 @@ __device__ __forceinline__ void flush_segments32(const SingleArgs &a, int par, i
 __device__ __forceinline__ void derive_penalties(const Sm &sm, int n)
 {
     const double r1 = sm.rho[0], r2 = sm.rho[1], r3 = sm.rho[2], r4 = sm.rho[3];
-    sm.bc[3] = r2 / (r1 + (double)n * r2); // kappa of step (b)
+    sm.bc[3] = r2 / fma((double)n, r2, r1); // kappa of step (b)
     sm.bc[4] = 0.5 * r3;
     sm.bc[5] = 0.5 * r4;
     sm.bc[6] = 0.5 * r1;
@@ -669,7 +639,7 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
                     sm.x0[i * q + j] = x0;
                     sum = j == lane ? d : sum + d;
                 }
-                const double x1n = warp_sum(sum) * iq64;              // (c), the mean over j
+                const double x1n = __dmul_rn(warp_sum(sum), iq64);    // (c), the mean over j
                 for (int j = lane; j < q; j += 32) {
                     const int pr = i * q + j;
                     const double d = x1n - sm.x0[pr], nun = sm.nu[pr] + d; // (h)
@@ -710,7 +680,8 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
             }
             const double lam = sm.lam[pr], zeta = sm.zeta[pr], hh = sm.h[pr], pp = sm.p[pr];
             const double W = fma(-nd, lam, S + g0s);                  // 1'(g(x) - lambda)
-            const double lamn = kappa * ((hh + pp) - W);              // (b) + (g)
+            const double lamn = __dmul_rn(kappa, (hh + pp) - W);      // (b) + (g); never fused into later sums,
+                                                                      // which a resumed solve forms from lamn
             const double Z = fma(nd, lamn, W);                        // 1'z
             const double hn = min_ord(Z - pp, ci);                    // (d)
             const double e = hn - Z, zn = lamn - lam;
