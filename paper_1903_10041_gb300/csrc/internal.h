@@ -10,6 +10,8 @@ namespace admm_impl {
 
 constexpr int kBlock = 256;          // threads per CTA of the mixed-precision solve kernel
 constexpr int kBlockF64 = 384;       // threads per CTA of the FP64 solve kernel
+constexpr int kBlockF64Cluster = 128; // the same of its cluster variant
+constexpr int kClusterCtas = 8;      // most CTAs of a cluster variant (the portable cluster size)
 constexpr int kSingleWarpsMax = 12;  // most warps per CTA of the single-instance kernels
 constexpr int kMaxM = ADMM_MAX_M;
 constexpr int kInfo = 16;            // doubles of the per-solve info record
@@ -72,7 +74,8 @@ struct SingleArgs {
 };
 
 // Launch the persistent single-instance solve kernel (cooperative launch);
-// minb selects the register-budget variant (1 or 2 CTAs per SM).
+// minb selects the register-budget variant (1 or 2 CTAs per SM), or the cluster
+// variant (0: all CTAs one thread-block cluster, no cooperative launch).
 cudaError_t launch_single(int precision, int minb, const SingleArgs &a, size_t smem, cudaStream_t st);
 // Max co-resident CTAs per SM of that kernel for the given dynamic smem.
 int single_blocks_per_sm(int precision, int m, int minb, size_t smem);
@@ -99,7 +102,9 @@ size_t single_smem_bytes(int m, int q, int precision);
 // Index of the kernel variant used for m sources (template bound).
 int single_mbound(int m);
 // Threads per CTA of the single-instance kernel of a precision.
-int single_threads(int precision);
+int single_threads(int precision, int minb);
+// The cluster variants (single_cluster.cu).
+void *single_cluster_fn(int precision, int m);
 // Row copies with conversion (device to device): rows x n values from a
 // source with row stride sld into a destination with row stride dld.
 void convert_rows_f32_to_f64(double *dst, int64_t dld, const float *src, int64_t sld, int n, int64_t rows,

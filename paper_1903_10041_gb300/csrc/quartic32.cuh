@@ -468,6 +468,26 @@ __device__ __forceinline__ bool newton_settled(float d0, float d1, float x)
     return a <= 1.0e-12f * s || (a <= 1.0e-10f * s && a <= 1.0e-5f * fabsf(d0));
 }
 
+// A certified root whose FP32 seed was too far off for two steps (a tiny b_2:
+// x is a small difference of numbers of size b_1 / b_2): Newton steps with FP64
+// slopes, which keep FP64's precision where the closed form loses it to that
+// difference (3.8e-10 at b_2 = 1e-6, b_1 = 1).  False: not settled either.
+static __device__ __noinline__ bool elem_refine64(Elem64 p, double &x)
+{
+    double y = x, last = INFINITY;
+    for (int t = 0; t < 8; ++t) {
+        const double w = fma(p.b2, y, p.b1), e = fma(w, y, -p.u), gp = fma(p.b2, y, w);
+        const double s = fma(p.hr1, fma(gp, gp, 2.0 * p.b2 * e), p.C);
+        if (!(s > 0.0)) return false;
+        const double d = fma(e * gp, p.hr1, fma(p.C, y, p.Dh)) / s;
+        y -= d;
+        if (fabs(d) <= 1.0e-15 * (fabs(y) + 1.0)) return x = y, true;
+        if (t > 3 && !(fabs(d) < 0.5 * last)) return false;
+        last = fabs(d);
+    }
+    return false;
+}
+
 // The constrained minimiser of an element with losses (b_2 or b_1 not zero).
 __device__ __forceinline__ double elem_min64_seeded(const Elem64 &p, float hr1f, double lo, double hi, int paper_mode)
 {
@@ -484,7 +504,7 @@ __device__ __forceinline__ double elem_min64_seeded(const Elem64 &p, float hr1f,
             x = fma(-H, r, x);
             d[t] = f64_to_f32_int(H) * rf;
         }
-        if (newton_settled(d[0], d[1], xf)) return clamp_ord(x, lo, hi);
+        if (newton_settled(d[0], d[1], xf) || elem_refine64(p, x)) return clamp_ord(x, lo, hi);
     }
     return elem_min64(p, lo, hi, paper_mode);
 }
