@@ -265,7 +265,7 @@ admm_status admm_quartic_min_f32(const float *A, const float *B, const float *C,
  * at zero, and calls that overlap on the GPU race on it, so the caller must
  * serialise them.  Instances whose scratch would exceed the array are
  * rejected with ADMM_EUNSUPPORTED (at most ADMM_MAX_PAIRS pairs on a
- * 152-SM GPU need under 200 KiB, so today the limit is not reached).  Only
+ * 152-SM GPU need under 300 KiB, so today the limit is not reached).  Only
  * ADMM_FP64 is available.  Returns as admm_solve, after the stream has
  * finished.  No cudaMalloc, cudaFree or other allocating call is made. */
 admm_status admm_solve_noalloc(const admm_problem *prob, const admm_params *params, admm_state *state,

@@ -259,7 +259,7 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
                     for (; v < v1; v += 32) {
                         const int kn = v + 32 < v1 ? (v + 32) * VW : -1;
                         vec32<M, VW, false, STAGE_ROLL>(ea, uoff, x1nu, j, v * VW, chk, cld, mud, rho1, rho3,
-                                                        rho4, iq, ghi, glo, fmx, fmn, fcr, fcs, esc, rec, stw, kn);
+                                                        rho4, iq, ghi, glo, fmx, fmn, fcr, fcs, esc, rec + 3, 4, stw, kn);
                     }
                     cp_async_wait0();
                 } else if constexpr (STG) {
@@ -277,14 +277,14 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
                         cp_async_commit();
                         cp_async_wait1(); // this round's copies have landed
                         vec32<M, VW, false, STAGE_DOUBLE>(ea, uoff, x1nu, j, v * VW, chk, cld, mud, rho1, rho3,
-                                                          rho4, iq, ghi, glo, fmx, fmn, fcr, fcs, esc, rec, cur);
+                                                          rho4, iq, ghi, glo, fmx, fmn, fcr, fcs, esc, rec + 3, 4, cur);
                     }
                     cp_async_wait0();
                 } else {
                     for (; v < v1; v += 32) {
                         if (v + 32 < v1) prefetch_vec32<M>(ea, j, (v + 32) * VW, cld);
                         vec32<M, VW, false>(ea, uoff, x1nu, j, v * VW, chk, cld, mud, rho1, rho3, rho4, iq, ghi,
-                                            glo, fmx, fmn, fcr, fcs, esc, rec);
+                                            glo, fmx, fmn, fcr, fcs, esc, rec + 3, 4);
                     }
                 }
             };

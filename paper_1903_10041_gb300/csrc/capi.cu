@@ -513,7 +513,7 @@ admm_status admm_create(const admm_problem *P, const admm_params *prm, admm_hand
     h->grid = sh.grid;
     h->nbmax = sh.nbmax;
     h->minb = sh.minb;
-    TRY(dev_malloc(af, &h->part, sizeof(double) * 2 * (size_t)q * h->nbmax * m * 4));
+    TRY(dev_malloc(af, &h->part, sizeof(double) * single_part_doubles(m, q, h->nbmax)));
     TRY(dev_malloc(af, &h->cpart, sizeof(double) * 2 * (size_t)h->grid * 4));
     st = reset_state(h);
     if (st != ADMM_OK) return bail(st);

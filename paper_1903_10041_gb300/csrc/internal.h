@@ -59,8 +59,8 @@ struct SingleArgs {
     void *x, *s, *mu;          // state arrays (storage type)
     void *s_lo, *mu_lo;        // mixed: low parts of the float-float column state s, mu
     double *scal;              // scalar state, in/out
-    double *part;              // [2][q][nbmax][m][4] partial records (gsum, dmax, dmin, x0), row-major by
-                               // row j and position b - b0(j) of the CTA among those touching row j
+    double *part;              // partial records of the rows by position of the CTA among those touching the
+                               // row (see Recs): single_part_doubles values
     double *cpart;             // [2][grid][4] per-CTA column maxima and objective partials
     unsigned *bar;             // barrier counter (zeroed before the launch)
     int *status;               // 0 or an admm_status set by a device wait
@@ -72,6 +72,14 @@ struct SingleArgs {
     int max_iter, check_every, xmin_mode, sweep, adapt;
     long long spin_ns;         // bound of one barrier wait
 };
+
+// Doubles rounded up to whole 32-byte sectors (a pair's records).
+inline __host__ __device__ int record_pad(int n) { return (n + 3) / 4 * 4; }
+// Doubles of SingleArgs::part: two parities of three planes [q][m][record_pad] and x at k = 0.
+inline size_t single_part_doubles(int m, int q, int nbmax)
+{
+    return 2 * (3 * (size_t)q * m * record_pad(nbmax) + record_pad(q * m));
+}
 
 // Launch the persistent single-instance solve kernel (cooperative launch);
 // minb selects the register-budget variant (1 or 2 CTAs per SM), or the cluster

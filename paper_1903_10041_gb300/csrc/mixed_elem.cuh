@@ -285,8 +285,8 @@ __device__ __forceinline__ void st2(float *p, float2 v) { *(float2 *)p = v; }
 // x1 + nu (read at k = 0 only) of pair pr, rounded to FP32 once per
 // iteration by the caller, so no FP64 operation runs per element.  The capacity
 // sums accumulate per lane in ghi/glo (the caller combines the lanes), the
-// D_k extrema in dmx/dmn.  rec (if k0 == 0) receives x at k = 0 as an FP32
-// value in the first four bytes of its slot (the scalar phase widens it).
+// D_k extrema in dmx/dmn.  rec[i rstep] (if k0 == 0) receives x at k = 0 as an
+// FP32 value in its first four bytes (the scalar phase widens it).
 // STAGE_ROLL: the inputs come from the lane's rolling stage stg, and each slot
 // group is refilled with the pair k0n (if >= 0) as soon as it is read.  The
 // first column is always < n; the second may be padding (k0 + 1 = n), and
@@ -299,7 +299,7 @@ template <int M, int VW, bool C64, int STAGE = STAGE_NONE, class EA>
 __device__ __forceinline__ void vec32(const EA &a, const float *uoff, const float *x1nu,
                                       int j, int k0, bool check, bool cold, float mu_div, float rho1, float rho3,
                                       float rho4, float iq, float2 *ghi, float2 *glo, float *dmx, float *dmn,
-                                      float &cm_r, float &cm_s, unsigned &esc, double *rec,
+                                      float &cm_r, float &cm_s, unsigned &esc, double *rec, int rstep,
                                       float2 *stg = nullptr, int k0n = -1)
 {
     static_assert(VW == 2, "the element update works on column pairs");
@@ -375,7 +375,7 @@ __device__ __forceinline__ void vec32(const EA &a, const float *uoff, const floa
             sx = ff2_addf(sx, xn); // sum_i x of (e), (f) in source order
             if (check) dx = ff2_add(dx, ff2_two_sum(xn, neg2(x0)));
             st2(a.x + a.xe(i, j, k0), xn);
-            if (k0 == 0) *(float *)(rec + i * 4 + 3) = xn.x; // FP32 in the slot; widened by the reader
+            if (k0 == 0) *(float *)(rec + i * rstep) = xn.x; // FP32 in the slot; widened by the reader
             float2 ghh, gll;
             g_ff2(b2, b1, xn, ghh, gll);
             if (!v1) {

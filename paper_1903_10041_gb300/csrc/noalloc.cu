@@ -215,7 +215,7 @@ extern "C" admm_status admm_solve_noalloc(const admm_problem *P, const admm_para
     const int grid = sh.grid, nbmax = sh.nbmax;
     // scratch layout (doubles, each region 32-double aligned)
     auto al = [](size_t v) { return (v + 31) / 32 * 32; };
-    const size_t n_part = al((size_t)2 * q * nbmax * m * 4), n_cpart = al((size_t)2 * grid * 4);
+    const size_t n_part = al(single_part_doubles(m, q, nbmax)), n_cpart = al((size_t)2 * grid * 4);
     const size_t n_scal = al((size_t)scal_size(m, q)), n_sumg0 = al((size_t)mq), n_info = al(kInfo), n_words = 32;
     const size_t need = n_part + n_cpart + n_scal + n_sumg0 + n_info + n_words;
     if (need > kScratchDoubles) {

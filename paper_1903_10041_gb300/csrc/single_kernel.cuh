@@ -144,7 +144,7 @@ struct Iter64 {
 template <int M>
 __device__ __forceinline__ void column64(const SingleArgs &a, const Sm &sm, const Iter64 &ic, int j, int k, bool check,
                                          bool cold, double mu_div, double *gs, double *dmx, double *dmn,
-                                         double &cm_r, double &cm_s, double *rec)
+                                         double &cm_r, double &cm_s, double *rec, int rstep)
 {
     const int m = a.m, q = a.q, ld = a.ld;
     const double *F2 = (const double *)a.f2, *F1 = (const double *)a.f1;
@@ -209,7 +209,7 @@ __device__ __forceinline__ void column64(const SingleArgs &a, const Sm &sm, cons
             if (jac) pre = i == 0 ? xt[i] : pre + xt[i];
             else pre = sx;
             X[((size_t)i * q + j) * ld + k] = xn;
-            if (k == 0) rec[i * 4 + 3] = xn;
+            if (k == 0) rec[i * rstep] = xn;
         }
     }
     const double v = (sx - yv) - mu;
@@ -318,11 +318,48 @@ __device__ __forceinline__ void row_ctas(const SingleArgs &a, int j, int &first,
     cnt = (int)((rbeg + a.rs - 1) / a.chunk) - first + 1;
 }
 
-// Partial record of row j written by this CTA (position among the CTAs
-// touching row j, in column order).
-__device__ __forceinline__ double *seg_record(const SingleArgs &a, const Sm &sm, int par, int j)
+// Records of one iteration parity: planes of S = sum g, max D and min D,
+// each [q][m][nbp] with a pair's records contiguous in the CTAs touching the
+// row, then x at k = 0 as [m][q].  The scalar phase of every CTA reads them
+// all, so what counts is the number of 32-byte sectors: with the records of
+// one CTA contiguous instead, each sector held one wanted value (n = 1e5, m =
+// 4, q = 20: 79.5 -> 76.1 us per iteration; n = 1000, q = 50 PHEV mixed 7.5 ->
+// 6.1, FP64 12.2 -> 11.4; n = 10007, m = 6, q = 11: 23.5 -> 21.5).
+struct Recs {
+    double *s;      // plane of S; the others follow at + plane
+    size_t plane;   // q m nbp
+    int m, nbp;
+    __device__ __forceinline__ size_t at(int i, int j, int t) const { return ((size_t)j * m + i) * nbp + t; }
+    __device__ __forceinline__ double *x0() const { return s + 3 * plane; }
+};
+__device__ __forceinline__ Recs records(const SingleArgs &a, int par)
 {
-    return a.part + ((size_t)(par * a.q + j) * a.nbmax + ((int)blockIdx.x - sm.rfirst[j])) * a.m * 4;
+    Recs r;
+    r.m = a.m;
+    r.nbp = record_pad(a.nbmax);
+    r.plane = (size_t)a.q * a.m * r.nbp;
+    r.s = a.part + (size_t)par * (3 * r.plane + record_pad(a.q * a.m)); // 32-byte aligned, as the pairs are
+    return r;
+}
+// Writes this CTA's record of (row j, source i); lo, hi on check iterations.
+template <bool CL>
+__device__ __forceinline__ void put_record(const SingleArgs &a, const Sm &sm, int par, int j, int i, double v, bool check,
+                                           double hi, double lo)
+{
+    if constexpr (CL) {
+        double *rec = sm.crec + (par * kMaxM + i) * 4;
+        rec[0] = v;
+        rec[1] = hi;
+        rec[2] = lo;
+    } else {
+        const Recs r = records(a, par);
+        const size_t e = r.at(i, j, (int)blockIdx.x - sm.rfirst[j]);
+        r.s[e] = v;
+        if (check) {
+            r.s[r.plane + e] = hi;
+            r.s[2 * r.plane + e] = lo;
+        }
+    }
 }
 
 // Reduction of one pass of row segments into their partial records, and (on
@@ -375,12 +412,7 @@ __device__ __forceinline__ void flush_segments(const SingleArgs &a, int par, int
             }
         }
         if (hl == 0 && t < ns * m) {
-            double *rec = CL ? sm.crec + par * kMaxM * 4 : seg_record(a, sm, par, jb + sg);
-            rec[i * 4 + 0] = r;
-            if (check) {
-                rec[i * 4 + 1] = hi;
-                rec[i * 4 + 2] = lo;
-            }
+            put_record<CL>(a, sm, par, jb + sg, i, r, check, hi, lo);
         }
     }
 }
@@ -443,12 +475,8 @@ __device__ __forceinline__ void flush_segments32(const SingleArgs &a, int par, i
             }
         }
         if (hl == 0 && t < ns * m) {
-            double *rec = CL ? sm.crec + par * kMaxM * 4 : seg_record(a, sm, par, jb + sg);
-            rec[i * 4 + 0] = f32_to_f64_int(r.hi) + f32_to_f64_int(r.lo);
-            if (check) {
-                rec[i * 4 + 1] = f32_to_f64_int(hi);
-                rec[i * 4 + 2] = f32_to_f64_int(lo);
-            }
+            put_record<CL>(a, sm, par, jb + sg, i, f32_to_f64_int(r.hi) + f32_to_f64_int(r.lo), check,
+                           f32_to_f64_int(hi), f32_to_f64_int(lo));
         }
     }
 }
@@ -501,7 +529,7 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
     const float iq = 1.0f / (float)q;
     // lanes that share the records of one pair in the scalar phase
     int gsh = 0;
-    while ((2 << gsh) <= a.nbmax && gsh < 5 && (mq << (gsh + 1)) <= NT) ++gsh;
+    while ((CL ? 2 : 4) << gsh <= a.nbmax && gsh < 5 && (mq << (gsh + 1)) <= NT) ++gsh;
     const int G = 1 << gsh;
     bool cold = sm.flags[0] != 0.0;
     double mu_div = sm.flags[1];
@@ -545,7 +573,9 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
             if (jb > jf) __syncthreads(); // the previous pass has been reduced
             const SegPlan sp = jb == jf ? sp0 : seg_plan<NWP>(c0, c1, rs, jb, jb + ns - 1, threadIdx.x >> 5);
             const int j = sp.j;
-            double *rec = CL ? sm.crec + par * kMaxM * 4 : seg_record(a, sm, par, j);
+            // x of source i at k = 0 goes to rec[i * rstep]
+            double *rec = CL ? sm.crec + par * kMaxM * 4 + 3 : records(a, par).x0() + j;
+            const int rstep = CL ? 4 : q;
             // row-local column range of the segment (k), and this thread's start and step
             const int kb = sp.kb, ke = sp.ke;
             const int first = sp.lw * 32 + (threadIdx.x & 31), stride = sp.nw * 32;
@@ -558,7 +588,7 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
                     dmn[i] = INFINITY;
                 }
                 for (int k = kb + first; k < ke; k += stride)
-                    column64<M>(a, sm, ic, j, k, check, cold, mu_div, gs, dmx, dmn, cm_r, cm_s, rec);
+                    column64<M>(a, sm, ic, j, k, check, cold, mu_div, gs, dmx, dmn, cm_r, cm_s, rec, rstep);
                 flush_segments<M, NWP, CL>(a, par, jb, ns, gs, dmx, dmn, cm_r, cm_s, check, m, sp, sm);
             } else {
                 float2 ghi[M], glo[M]; // per-lane capacity sums of the column pairs
@@ -599,7 +629,7 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
                             const int k0n = k0 + stride * VW < kn ? k0 + stride * VW : -1;
                             vec32<M, VW, PREC == ADMM_MIXED_FP64CUBIC, STAGE_ROLL>(
                                 ea, sm.uoff, sm.x1nu, j, k0, chk, cld, mud, rho1, rho3, rho4, iq, ghi, glo,
-                                fmx, fmn, fcr, fcs, esc, rec, stw, k0n);
+                                fmx, fmn, fcr, fcs, esc, rec, rstep, stw, k0n);
                         }
                         cp_async_wait0();
                     } else {
@@ -608,7 +638,7 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
                                 if (k0 + stride * VW < kn) prefetch_vec32<M>(ea, j, k0 + stride * VW, cld);
                             vec32<M, VW, PREC == ADMM_MIXED_FP64CUBIC>(ea, sm.uoff, sm.x1nu, j, k0, chk, cld,
                                                                        mud, rho1, rho3, rho4, iq, ghi, glo,
-                                                                       fmx, fmn, fcr, fcs, esc, rec);
+                                                                       fmx, fmn, fcr, fcs, esc, rec, rstep);
                         }
                     }
                 };
@@ -648,27 +678,22 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
         // per iteration (us): n = 1000, q = 50 PHEV FP64 16.7 -> 12.1, mixed
         // 10.0 -> 7.7; n = 4099, m = 3, q = 7 FP64 23.3 -> 15.2; n = 10007, m = 6,
         // q = 11 mixed 31.4 -> 24.0; n = 100 FP64 1.8x.
-        const size_t rstride = (size_t)m * 4;
-        const double *prec = CL ? sm.crec + par * kMaxM * 4 : a.part + (size_t)par * q * a.nbmax * rstride;
-        // entry e of source i in record t of row j (the cluster variant's CTA j * pieces + t holds it)
-        auto record = [&](int j, int t, int i, int e) {
-            if constexpr (CL) {
-                const double *p = prec + i * 4 + e;
-                return a.grid == 1 ? p : (const double *)cg::this_cluster().map_shared_rank((double *)p, j * a.pieces + t);
-            } else {
-                return prec + ((size_t)j * a.nbmax + t) * rstride + i * 4 + e;
-            }
+        const Recs rr = records(a, par);
+        // the cluster variant's records: CTA j * pieces + t holds record t of row j
+        auto remote = [&](int j, int t, int i, int e) {
+            const double *p = sm.crec + (par * kMaxM + i) * 4 + e;
+            return a.grid == 1 ? p : (const double *)cg::this_cluster().map_shared_rank((double *)p, j * a.pieces + t);
         };
-        auto rd = [](const double *p) { return CL ? *p : __ldcg(p); };
         double r1m = 0.0, r2m = 0.0, r3m = 0.0, r4m = 0.0, s1m = 0.0, s2m = 0.0, s3m = 0.0;
         {
             const int lane = threadIdx.x & 31;
             for (int i = NWP - 1 - (int)(threadIdx.x >> 5); i < m; i += NWP) {
                 double sum = 0.0;
                 for (int j = lane; j < q; j += 32) {
-                    // x at k = 0: FP64 in the FP64 kernel, FP32 in the first four bytes of the slot in the mixed ones
-                    const double *r0 = record(j, 0, i, 3);
-                    const double x0 = MIXED ? f32_to_f64_int(CL ? *(const float *)r0 : __ldcg((const float *)r0)) : rd(r0);
+                    // x at k = 0: FP64 in the FP64 kernel, FP32 in the slot's first four bytes in the mixed ones
+                    double x0;
+                    if constexpr (CL) x0 = MIXED ? f32_to_f64_int(*(const float *)remote(j, 0, i, 3)) : *remote(j, 0, i, 3);
+                    else x0 = MIXED ? f32_to_f64_int(__ldcg((const float *)(rr.x0() + i * q + j))) : ldcg(rr.x0() + i * q + j);
                     const double d = x0 - sm.nu[i * q + j];
                     sm.x0[i * q + j] = x0;
                     sum = j == lane ? d : sum + d;
@@ -693,17 +718,32 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
             const int i = pr / q, j = pr - i * q;
             const int nb = sm.rcnt[j];
             const double g0s = a.sumg0[pr], ci = a.c[i];
-            // records of row j in CTA order, every G-th per lane; a fixed order of the sums
+            // records of row j, every G-th (pair) per lane; a fixed order of the sums
             double S = 0.0, dmx = -INFINITY, dmn = INFINITY;
-#pragma unroll 8
-            for (int t = sub; t < nb; t += G) {
-                const double *rec = record(j, t, i, 0);
-                const double v = rd(rec);
-                S = t == sub ? v : S + v;
-                if (check) {
-                    dmx = max_ord(dmx, rd(rec + 1));
-                    dmn = min_ord(dmn, rd(rec + 2));
+            if constexpr (CL) {
+                for (int t = sub; t < nb; t += G) {
+                    const double v = *remote(j, t, i, 0);
+                    S = t == sub ? v : S + v;
+                    if (check) {
+                        dmx = max_ord(dmx, *remote(j, t, i, 1));
+                        dmn = min_ord(dmn, *remote(j, t, i, 2));
+                    }
                 }
+            } else {
+                // two records per load, neighbouring lanes on neighbouring pairs of records; the
+                // padding past nb is not added
+                const double *rs = rr.s + rr.at(i, j, 0);
+#pragma unroll 4
+                for (int t = 2 * sub; t < nb; t += 2 * G) {
+                    const double2 v = __ldcg((const double2 *)(rs + t));
+                    const double w = t + 1 < nb ? v.x + v.y : v.x;
+                    S = t == 2 * sub ? w : S + w;
+                }
+                if (check)
+                    for (int t = sub; t < nb; t += G) {
+                        dmx = max_ord(dmx, ldcg(rs + rr.plane + t));
+                        dmn = min_ord(dmn, ldcg(rs + 2 * rr.plane + t));
+                    }
             }
             for (int o = G >> 1; o > 0; o >>= 1) {
                 S += __shfl_xor_sync(0xffffffffu, S, o);
@@ -740,8 +780,8 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
             for (int b = threadIdx.x; b < a.grid; b += NT) {
                 const double *cm = CL ? sm.ccm + par * 2 : a.cpart + ((size_t)par * a.grid + b) * 4;
                 if (CL && a.grid > 1) cm = cg::this_cluster().map_shared_rank((double *)cm, b);
-                r1m = max_nonneg(r1m, rd(cm));
-                s3m = max_nonneg(s3m, rd(cm + 1));
+                r1m = max_nonneg(r1m, CL ? cm[0] : ldcg(cm));
+                s3m = max_nonneg(s3m, CL ? cm[1] : ldcg(cm + 1));
             }
             double v[8] = {r1m, r2m, r3m, r4m, s1m, s2m, s3m, 0.0};
             auto mx = [](double k, double s, int o) { return max_nonneg(k, __shfl_xor_sync(0xffffffffu, s, o)); };
