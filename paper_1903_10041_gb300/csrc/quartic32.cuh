@@ -388,7 +388,7 @@ __device__ __forceinline__ bool elem_polish32(float b2, float b1, float u, float
     const float s = fmaf(hr1, fmaf(gp1, gp1, 2.0f * b2 * e1), C);
     x = y;
     r = rcp_fast(s);
-    return s > 0.0f && isfinite(x) && isfinite(r) && r >= 1.2e-38f;
+    return fabsf(x) < 1.0e30f && r >= 1.2e-38f && r < 1.0e38f;
 }
 
 // The minimiser's FP32 root where H has three real roots (Delta < 0
@@ -427,18 +427,19 @@ static __device__ __noinline__ bool elem_trig32(float Q, float R, float dR, floa
 // FP32 root of H (x) and 1 / H'(x) (r) that the minimiser is refined from:
 // the quadratic case (b_2 = 0), the Cardano branch with Delta > 0 certified,
 // and the trig branch with Delta < 0 certified where elem_trig32 can tell the root.
-// Q and R carry the rounding of b_2, b_1, u, C, Dh to FP32, that of their own
-// operations and two reciprocals off by 2 ulp: |dQ| <= 24 v mQ, |dR| <= 17 v mR
-// (v = 2^-24, mQ, mR the sums of the terms' magnitudes), so |dDelta| <=
-// v (76 Q^2 mQ + 37 |R| mR); the bound takes 128 v for both.
-__device__ __forceinline__ bool elem_seed32(float b2, float b1, float u, float C, float Dh, float hr1, float lo,
-                                            float hi, int paper_mode, float &x, float &r)
+// Q and R carry the truncation of b_2, b_1, u, C, Dh to FP32 (2 v, v = 2^-24),
+// the rounding of their own operations and two reciprocals off by 2 ulp: |dQ|
+// <= 30 v mQ, |dR| <= 22 v mR (mQ, mR the sums of the terms' magnitudes), so
+// |dDelta| <= v (94 Q^2 mQ + 48 |R| mR); the bound takes 128 v for both.
+__device__ __forceinline__ bool elem_seed32(float b2, float b1, float u, float C, float Dh, float hr1, double lo,
+                                            double hi, int paper_mode, float &x, float &r)
 {
-    const float hb1 = hr1 * b1;
-    if (b2 == 0.0f) {
+    if (!(fabsf(b1) + fabsf(u) + C + fabsf(Dh) < 1.0e37f)) return false; // cut off at the end of the FP32 range
+    if (b2 <= 1.2e-38f) { // 0 (or below the FP32 range): the converted value is the smallest normal one
+        const float hb1 = hr1 * b1;
         r = rcp_fast(fmaf(hb1, b1, C));
         x = fmaf(hb1, u, -Dh) * r;
-        return isfinite(x) && r >= 1.2e-38f;
+        return fabsf(x) < 1.0e30f && r >= 1.2e-38f && r < 1.0e38f;
     }
     const float b3 = 0.5f * b1 * rcp_fast(b2);
     const float v = 0.5f * b1 * b3;                 // b_1^2 / (4 b_2)
@@ -454,7 +455,7 @@ __device__ __forceinline__ bool elem_seed32(float b2, float b1, float u, float C
         const float sq = sqrt_fast(Dl);
         const float S = cbrt_fast(R >= 0.0f ? R + sq : R - sq);
         y = S - Q * rcp_fast(S) - b3;
-    } else if (!(Dl < -bound) || !elem_trig32(Q, R, 2.0e-6f * mR, b3, lo, hi, paper_mode, y)) {
+    } else if (!(Dl < -bound) || !elem_trig32(Q, R, 2.0e-6f * mR, b3, f64_to_f32_seed(lo), f64_to_f32_seed(hi), paper_mode, y)) {
         return false;
     }
     return elem_polish32(b2, b1, u, C, Dh, hr1, y, x, r);
@@ -492,17 +493,17 @@ static __device__ __noinline__ bool elem_refine64(Elem64 p, double &x)
 __device__ __forceinline__ double elem_min64_seeded(const Elem64 &p, float hr1f, double lo, double hi, int paper_mode)
 {
     float xf, rf;
-    if (elem_seed32(f64_to_f32_int(p.b2), f64_to_f32_int(p.b1), f64_to_f32_int(p.u), f64_to_f32_int(p.C),
-                    f64_to_f32_int(p.Dh), hr1f, f64_to_f32_int(lo), f64_to_f32_int(hi), paper_mode, xf, rf)) {
-        const double r = f32_to_f64_int(rf);
-        double x = f32_to_f64_int(xf);
+    if (elem_seed32(f64_to_f32_seed(p.b2), f64_to_f32_seed(p.b1), f64_to_f32_seed(p.u), f64_to_f32_seed(p.C),
+                    f64_to_f32_seed(p.Dh), hr1f, lo, hi, paper_mode, xf, rf)) {
+        const double r = f32_to_f64_seed(rf);
+        double x = f32_to_f64_seed(xf);
         float d[2];
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
             const double w = fma(p.b2, x, p.b1), e = fma(w, x, -p.u), gp = fma(p.b2, x, w);
             const double H = fma(e * gp, p.hr1, fma(p.C, x, p.Dh));
             x = fma(-H, r, x);
-            d[t] = f64_to_f32_int(H) * rf;
+            d[t] = f64_to_f32_seed(H) * rf;
         }
         if (newton_settled(d[0], d[1], xf) || elem_refine64(p, x)) return clamp_ord(x, lo, hi);
     }
@@ -512,10 +513,10 @@ __device__ __forceinline__ double elem_min64_seeded(const Elem64 &p, float hr1f,
 // The same without losses: H(x) = C x + Dh.
 __device__ __forceinline__ double elem_min64_linear(double C, double Dh, double lo, double hi)
 {
-    const float Cf = f64_to_f32_int(C), rf = rcp_fast(Cf), xf = -f64_to_f32_int(Dh) * rf;
-    if (rf >= 1.2e-38f && isfinite(rf) && isfinite(xf)) {
-        const double r = f32_to_f64_int(rf);
-        double x = f32_to_f64_int(xf);
+    const float Cf = f64_to_f32_seed(C), rf = rcp_fast(Cf), xf = -f64_to_f32_seed(Dh) * rf;
+    if (rf >= 1.2e-38f && rf < 1.0e38f && fabsf(xf) < 1.0e30f) {
+        const double r = f32_to_f64_seed(rf);
+        double x = f32_to_f64_seed(xf);
         x = fma(-fma(C, x, Dh), r, x);
         x = fma(-fma(C, x, Dh), r, x);
         return clamp_ord(x, lo, hi);

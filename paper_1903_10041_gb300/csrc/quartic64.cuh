@@ -62,6 +62,21 @@ __device__ __forceinline__ double f32_to_f64_int(float v)
     const bool z = a < 0x00800000u;
     return __hiloint2double((int)((b & 0x80000000u) | (z ? 0u : (a >> 3) + (896u << 20))), (int)(z ? 0u : b << 29));
 }
+// (float)v truncated, half the instructions: for seeds, whose error bounds
+// count two units of 2^-24 per converted value.  Magnitudes outside the FP32
+// normal range (zero among them) give its ends.
+__device__ __forceinline__ float f64_to_f32_seed(double v)
+{
+    const int hi = __double2hiint(v);
+    const int a = min(max((hi & 0x7fffffff) - 0x38000000, 0x00100000), 0x0fefffff); // 8 exponent bits, 20 of the mantissa
+    return __uint_as_float(__funnelshift_l((unsigned)__double2loint(v), (unsigned)a, 3) | ((unsigned)hi & 0x80000000u));
+}
+// (double)v for a normal v; a zero gives 2^-127.
+__device__ __forceinline__ double f32_to_f64_seed(float v)
+{
+    const int b = __float_as_int(v);
+    return __hiloint2double((int)(((unsigned)(b >> 3) & 0x8fffffffu) + 0x38000000u), b << 29);
+}
 // Doubles as integers in the order of their values (no NaN; -0 before +0).
 __device__ __forceinline__ long long ord64(double v)
 {
