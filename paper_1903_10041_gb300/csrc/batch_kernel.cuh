@@ -532,7 +532,15 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
     sync_team(); // rank 0 has read every member's shared memory
 }
 
-template <int NW, int M, bool ROLL> __global__ void __launch_bounds__(NW * 32, 16 / NW) batch_kernel(BatchArgs a)
+// Registers: CTAs of 16 warps have 128 a thread; smaller ones take 255, which
+// leaves 8 warps per SM instead of 16 but nothing spilled.  With 8 warps per
+// CTA that is faster at every batch size tried, most where the largest
+// instances' iterations on one CTA are what a batch waits for (150 / 600 / 2000
+// instances x 100 iterations: 38.4 / 58.4 / 66.9 -> 22.4 / 37.7 / 57.1 ms).  12 warps
+// of 168 registers in the place of 16: 4096 adaptive solves 688 -> 673 ms, but a
+// burst of 48 served solves 106 -> 118 ms.
+template <int NW, int M, bool ROLL>
+__global__ void __launch_bounds__(NW * 32, NW == 16 ? 1 : 8 / NW) batch_kernel(BatchArgs a)
 {
     extern __shared__ double smem[];
     __shared__ int s_item;

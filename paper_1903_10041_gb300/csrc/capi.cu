@@ -173,7 +173,7 @@ struct admm_handle {
     double *info_host = nullptr; // pinned
     cudaEvent_t done = nullptr;  // recorded after each queued solve (admm_wait)
     // launch shape
-    int grid = 0, nbmax = 0, rs = 0, minb = 1;
+    int grid = 0, nbmax = 0, rs = 0, wide = 1;
     int64_t chunk = 0, ncols = 0;
     int pieces = 0;
     size_t smem = 0;
@@ -512,7 +512,7 @@ admm_status admm_create(const admm_problem *P, const admm_params *prm, admm_hand
     h->pieces = sh.pieces;
     h->grid = sh.grid;
     h->nbmax = sh.nbmax;
-    h->minb = sh.minb;
+    h->wide = sh.wide;
     TRY(dev_malloc(af, &h->part, sizeof(double) * single_part_doubles(m, q, h->nbmax)));
     TRY(dev_malloc(af, &h->cpart, sizeof(double) * 2 * (size_t)h->grid * 4));
     st = reset_state(h);
@@ -664,7 +664,7 @@ admm_status admm_solve(admm_handle *h, const admm_state *warm, admm_result *out,
     CUDA_TRY(cudaMemsetAsync(h->status, 0, sizeof(int), st));
     CUDA_TRY(cudaMemsetAsync(h->info + 15, 0, sizeof(double), st));
     a.dbg = (unsigned long long *)(h->info + 15);
-    CUDA_TRY(launch_single(h->prm.precision, h->minb, a, h->smem, st));
+    CUDA_TRY(launch_single(h->prm.precision, h->wide, a, h->smem, st));
     CUDA_TRY(cudaMemcpyAsync(h->info_host, h->info, kInfo * 8, cudaMemcpyDeviceToHost, st));
     if (out && out->x) CUDA_TRY(export_rows(h, out->x, out->on_device != 0, h->x, (int64_t)h->m * h->q, st));
     if (out && out->x1)

@@ -9,6 +9,7 @@
 namespace admm_impl {
 
 constexpr int kBlock = 256;          // threads per CTA of the mixed-precision solve kernel
+constexpr int kBlockWide = 384;      // the same where a thread has several columns
 constexpr int kBlockF64 = 384;       // threads per CTA of the FP64 solve kernel
 constexpr int kBlockF64Cluster = 128; // the same of its cluster variant
 constexpr int kClusterCtas = 8;      // most CTAs of a cluster variant (the portable cluster size)
@@ -82,11 +83,11 @@ inline size_t single_part_doubles(int m, int q, int nbmax)
 }
 
 // Launch the persistent single-instance solve kernel (cooperative launch);
-// minb selects the register-budget variant (1 or 2 CTAs per SM), or the cluster
-// variant (0: all CTAs one thread-block cluster, no cooperative launch).
-cudaError_t launch_single(int precision, int minb, const SingleArgs &a, size_t smem, cudaStream_t st);
+// wide selects the variant: 1, or 2 (mixed: more threads, for several columns per
+// thread), or 0 (all CTAs one thread-block cluster, no cooperative launch).
+cudaError_t launch_single(int precision, int wide, const SingleArgs &a, size_t smem, cudaStream_t st);
 // Max co-resident CTAs per SM of that kernel for the given dynamic smem.
-int single_blocks_per_sm(int precision, int m, int minb, size_t smem);
+int single_blocks_per_sm(int precision, int m, int wide, size_t smem);
 // Launch shape of a solve: CTAs, columns per CTA (a multiple of the vector
 // width in mixed precision), kernel variant, and the most CTAs touching one
 // row j (records per row).  grid = 0: the kernel cannot be resident.
@@ -94,7 +95,7 @@ struct SingleShape {
     int grid;
     int64_t chunk;
     int pieces;
-    int minb;
+    int wide;
     int nbmax;
 };
 
@@ -110,7 +111,7 @@ size_t single_smem_bytes(int m, int q, int precision);
 // Index of the kernel variant used for m sources (template bound).
 int single_mbound(int m);
 // Threads per CTA of the single-instance kernel of a precision.
-int single_threads(int precision, int minb);
+int single_threads(int precision, int wide);
 // The cluster variants (single_cluster.cu).
 void *single_cluster_fn(int precision, int m);
 // Row copies with conversion (device to device): rows x n values from a

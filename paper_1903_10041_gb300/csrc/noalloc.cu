@@ -302,7 +302,7 @@ extern "C" admm_status admm_solve_noalloc(const admm_problem *P, const admm_para
     a.sweep = prm->sweep;
     a.adapt = prm->adapt_rho;
     a.spin_ns = 2000000000LL;
-    e = launch_single(prm->precision, sh.minb, a, smem, cs);
+    e = launch_single(prm->precision, sh.wide, a, smem, cs);
     if (e != cudaSuccess) return nfail(ADMM_ECUDA, "solve launch: ", cudaGetErrorString(e));
     noalloc_finish<<<(mq + 255) / 256, 256, 0, cs>>>(m, q, scal, st->lam, st->zeta, st->h, st->p, st->nu, st->x1);
     double hinfo[kInfo], tail[6];

@@ -9,26 +9,26 @@ namespace admm_impl {
 
 namespace {
 
-template <int M> void *single_fn(int precision, int minb)
+template <int M> void *single_fn(int precision, int wide)
 {
     switch (precision) {
     case ADMM_MIXED:
-        return minb == 1 ? (void *)single_kernel<M, ADMM_MIXED, 1, kBlock, false>
-                         : (void *)single_kernel<M, ADMM_MIXED, 2, kBlock, false>;
+        return wide == 1 ? (void *)single_kernel<M, ADMM_MIXED, kBlock, false>
+                         : (void *)single_kernel<M, ADMM_MIXED, kBlockWide, false>;
     case ADMM_MIXED_FP64CUBIC:
-        return minb == 1 ? (void *)single_kernel<M, ADMM_MIXED_FP64CUBIC, 1, kBlock, false>
-                         : (void *)single_kernel<M, ADMM_MIXED_FP64CUBIC, 2, kBlock, false>;
-    default: return (void *)single_kernel<M, ADMM_FP64, 1, kBlockF64, false>;
+        return wide == 1 ? (void *)single_kernel<M, ADMM_MIXED_FP64CUBIC, kBlock, false>
+                         : (void *)single_kernel<M, ADMM_MIXED_FP64CUBIC, kBlockWide, false>;
+    default: return (void *)single_kernel<M, ADMM_FP64, kBlockF64, false>;
     }
 }
 
-void *pick(int precision, int m, int minb)
+void *pick(int precision, int m, int wide)
 {
-    if (minb == 0) return single_cluster_fn(precision, m);
+    if (wide == 0) return single_cluster_fn(precision, m);
     switch (single_mbound(m)) {
-    case 2: return single_fn<2>(precision, minb);
-    case 4: return single_fn<4>(precision, minb);
-    default: return single_fn<8>(precision, minb);
+    case 2: return single_fn<2>(precision, wide);
+    case 4: return single_fn<4>(precision, wide);
+    default: return single_fn<8>(precision, wide);
     }
 }
 
@@ -38,11 +38,12 @@ int single_mbound(int m) { return m <= 2 ? 2 : (m <= 4 ? 4 : 8); }
 
 // FP64: 12 warps (one CTA per SM, up to 168 registers a thread); the FP64
 // units are shared by the SM, so more warps hide more of their latency.
-// The cluster variant (minb = 0) takes a column per thread on one warp per
+// The cluster variant (wide = 0) takes a column per thread on one warp per
 // scheduler: fewer warps make its barriers cheaper.
-int single_threads(int precision, int minb)
+int single_threads(int precision, int wide)
 {
-    return precision != ADMM_FP64 ? kBlock : (minb == 0 ? kBlockF64Cluster : kBlockF64);
+    if (precision != ADMM_FP64) return wide == 2 ? kBlockWide : kBlock;
+    return wide == 0 ? kBlockF64Cluster : kBlockF64;
 }
 
 // Launch configuration of the cluster variant: one cluster of `ctas` CTAs.
@@ -66,17 +67,17 @@ size_t single_smem_bytes(int m, int q, int precision)
     const int mb = single_mbound(m);
     size_t stage = 0; // the rolling stage of the mixed kernels, one per warp
     if (precision != ADMM_FP64 && mb <= 4)
-        stage = (size_t)(kBlock / 32) * (mb == 2 ? roll_slots<2>() : roll_slots<4>()) * 32 * sizeof(float2);
+        stage = (size_t)(kBlockWide / 32) * (mb == 2 ? roll_slots<2>() : roll_slots<4>()) * 32 * sizeof(float2);
     return single_carve_bytes(m, q) + stage;
 }
 
-int single_blocks_per_sm(int precision, int m, int minb, size_t smem)
+int single_blocks_per_sm(int precision, int m, int wide, size_t smem)
 {
-    void *fn = pick(precision, m, minb);
+    void *fn = pick(precision, m, wide);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return 0;
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, single_threads(precision, minb), smem) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, single_threads(precision, wide), smem) != cudaSuccess)
         return 0;
     return nb;
 }
@@ -111,7 +112,7 @@ SingleShape single_shape(int precision, int m, int q, int64_t rs, int nsm, size_
         const int64_t cap = mixed ? (int64_t)kBlock * unit : kBlockF64Cluster;
         const int64_t p = (rs + cap - 1) / cap;
         if (q * p <= kClusterCtas && cluster_resident(precision, m, (int)(q * p), smem)) {
-            sh.minb = 0;
+            sh.wide = 0;
             sh.pieces = (int)p;
             sh.grid = (int)(q * p);
             sh.nbmax = (int)p;
@@ -122,10 +123,10 @@ SingleShape single_shape(int precision, int m, int q, int64_t rs, int nsm, size_
     // Contiguous equal column chunks over as many SMs as there are warps of
     // work (FP64 throughput per SM is the scarce resource), one CTA per SM
     // while that covers every column vector in a single pass, two otherwise.
-    sh.minb = (mixed && ncols > (int64_t)nsm * single_threads(precision, 1) * unit) ? 2 : 1;
-    int per_sm = single_blocks_per_sm(precision, m, sh.minb, smem);
-    if (per_sm < 1 && sh.minb == 2) {
-        sh.minb = 1;
+    sh.wide = (mixed && ncols > (int64_t)nsm * single_threads(precision, 1) * unit) ? 2 : 1;
+    int per_sm = single_blocks_per_sm(precision, m, sh.wide, smem);
+    if (per_sm < 1 && sh.wide == 2) {
+        sh.wide = 1;
         per_sm = single_blocks_per_sm(precision, m, 1, smem);
     }
     if (per_sm < 1) return sh;
@@ -156,20 +157,20 @@ SingleShape single_shape(int precision, int m, int q, int64_t rs, int nsm, size_
     return sh;
 }
 
-cudaError_t launch_single(int precision, int minb, const SingleArgs &a, size_t smem, cudaStream_t st)
+cudaError_t launch_single(int precision, int wide, const SingleArgs &a, size_t smem, cudaStream_t st)
 {
-    void *fn = pick(precision, a.m, minb);
+    void *fn = pick(precision, a.m, wide);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     SingleArgs copy = a;
     void *args[] = {(void *)&copy};
-    if (minb == 0) {
+    if (wide == 0) {
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
         cluster_config(cfg, attr, precision, a.grid, smem, st);
         return cudaLaunchKernelExC(&cfg, fn, args);
     }
-    return cudaLaunchCooperativeKernel(fn, dim3(a.grid), dim3(single_threads(precision, minb)), args, smem, st);
+    return cudaLaunchCooperativeKernel(fn, dim3(a.grid), dim3(single_threads(precision, wide)), args, smem, st);
 }
 
 } // namespace admm_impl

@@ -8,9 +8,9 @@ namespace {
 template <int M> void *cluster_fn(int precision)
 {
     switch (precision) {
-    case ADMM_MIXED: return (void *)single_kernel<M, ADMM_MIXED, 1, kBlock, true>;
-    case ADMM_MIXED_FP64CUBIC: return (void *)single_kernel<M, ADMM_MIXED_FP64CUBIC, 1, kBlock, true>;
-    default: return (void *)single_kernel<M, ADMM_FP64, 1, kBlockF64Cluster, true>;
+    case ADMM_MIXED: return (void *)single_kernel<M, ADMM_MIXED, kBlock, true>;
+    case ADMM_MIXED_FP64CUBIC: return (void *)single_kernel<M, ADMM_MIXED_FP64CUBIC, kBlock, true>;
+    default: return (void *)single_kernel<M, ADMM_FP64, kBlockF64Cluster, true>;
     }
 }
 } // namespace

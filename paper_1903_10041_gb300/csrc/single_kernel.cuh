@@ -496,11 +496,15 @@ __device__ __forceinline__ void derive_penalties(const Sm &sm, int n)
     f[3] = (float)(0.5 * r1);
 }
 
-// MINB: CTAs per SM the register budget is sized for.  FP64 takes 1 (its
-// element update needs about 250 registers); the mixed kernel comes in both:
-// 1 for problems that fill at most one CTA per SM (no spills), 2 otherwise.
-template <int M, int PREC, int MINB, int NT, bool CL>
-__global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
+// NT: threads of a CTA, one CTA per SM.  FP64 takes 384 (168 registers).  The
+// mixed kernel takes 256 (255 registers, no spills) where one pass covers the
+// columns, and 384 where a thread has several: two CTAs of 256 at 128
+// registers keep a third more warps but spill, and the reloads come back
+// through an L1 that the stage's copies sweep (n = 1e5, m = 4, q = 20: 76.1 ->
+// 66.7 us per iteration; 320 threads 72.3, 448 79.5; n = 10007, m = 6, q = 11:
+// 21.5 -> 18.8).
+template <int M, int PREC, int NT, bool CL>
+__global__ void __launch_bounds__(NT, 1) single_kernel(SingleArgs a)
 {
     namespace cg = cooperative_groups;
     constexpr int NWP = NT / 32;
@@ -634,7 +638,7 @@ __global__ void __launch_bounds__(NT, MINB) single_kernel(SingleArgs a)
                         cp_async_wait0();
                     } else {
                         for (int k0 = kb + first * VW; k0 < kn; k0 += stride * VW) {
-                            if constexpr (MINB == 2) // several vectors per thread: fetch the next one into L2
+                            if constexpr (NT > kBlock) // several vectors per thread: fetch the next one into L2
                                 if (k0 + stride * VW < kn) prefetch_vec32<M>(ea, j, k0 + stride * VW, cld);
                             vec32<M, VW, PREC == ADMM_MIXED_FP64CUBIC>(ea, sm.uoff, sm.x1nu, j, k0, chk, cld,
                                                                        mud, rho1, rho3, rho4, iq, ghi, glo,
