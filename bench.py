@@ -98,7 +98,8 @@ NCU_TRAFFIC_BATCH = {"bytes_per_element_iter": (1811961266176 + 614259118080) / 
 NCU_FP64_PIPE = {("phev n=1000 q=50", "fp64"): {"pct": 60.47, "src": "0f1fa41955024aab"}}
 
 # Sources each solve kernel is compiled from.
-SINGLE_KERNEL_SOURCES = ("single.cu", "quartic32.cuh", "quartic64.cuh", "mixed_elem.cuh", "common.cuh", "internal.h")
+SINGLE_KERNEL_SOURCES = ("single.cu", "single_cluster.cu", "single_kernel.cuh", "quartic32.cuh", "quartic64.cuh",
+                         "mixed_elem.cuh", "common.cuh", "internal.h")
 BATCH_KERNEL_SOURCES = ("batch_kernel.cuh", "batch_w4.cu", "batch_w8.cu", "batch_w16.cu", "batch.h", "quartic32.cuh",
                         "quartic64.cuh", "mixed_elem.cuh", "common.cuh", "internal.h")
 

@@ -142,23 +142,22 @@ static __device__ __noinline__ int cubic_branch64(float A, float B, float C, flo
 __device__ __forceinline__ float quartic_min32(float A, float B, float C, float D, float lo, float hi,
                                                int paper_mode, unsigned &esc)
 {
-    // Every operation below is rounded as the packed path (quartic_min32x2)
-    // rounds it, so a lane gets the same bits on either path.
     if (A == 0.0f) return clampf(__fmul_rn(-D, rcp_fast(__fadd_rn(C, C))), lo, hi);
+    // unfused, so that an input near a double root or a tie keeps the rounding it always had
     const float inv = rcp_fast(A);
     const float b = __fmul_rn(__fmul_rn(0.75f, B), inv);
     const float c = __fmul_rn(__fmul_rn(0.5f, C), inv);
     const float d = __fmul_rn(__fmul_rn(0.25f, D), inv);
     const float b3 = __fmul_rn(b, 1.0f / 3.0f);
-    const float b3s = __fmul_rn(b3, b3);
+    const float b3s = __fmul_rn(b3, b3), b3c = __fmul_rn(b3s, b3);
     const float Q = __fmaf_rn(c, 1.0f / 3.0f, -b3s);
-    const float hc = __fmul_rn(0.5f, c), hd = __fmul_rn(0.5f, d);
-    const float R = __fmaf_rn(b3, __fsub_rn(hc, b3s), -hd);
+    const float bhc = __fmul_rn(b3, __fmul_rn(0.5f, c));
+    const float R = __fsub_rn(__fsub_rn(bhc, b3c), __fmul_rn(0.5f, d));
     const float Qs = __fmul_rn(Q, Q);
-    const float Dl = __fmaf_rn(Qs, Q, __fmul_rn(R, R));
+    const float Dl = __fadd_rn(__fmul_rn(Qs, Q), __fmul_rn(R, R));
     // magnitudes entering Q, R (including the rounding of b, c, d); |Q| <= mQ and |R| <= mR
     const float mQ = __fmaf_rn(fabsf(c), 1.0f / 3.0f, b3s);
-    const float mR = __fmaf_rn(fabsf(b3), __fadd_rn(b3s, fabsf(hc)), fabsf(hd));
+    const float mR = __fmaf_rn(0.5f, fabsf(d), __fadd_rn(fabsf(bhc), fabsf(b3c)));
     // |fl(Delta) - Delta| <= u (78 Q^2 mQ + 12 |Q|^3 + 88 |R| mR + 4 R^2) with u = 2^-24
     // (a factor 2 over the first-order propagation of the roundings above,
     // with a reciprocal of A off by up to 2 ulp).  As |Q|^3 <= Q^2 mQ and
@@ -177,8 +176,8 @@ __device__ __forceinline__ float quartic_min32(float A, float B, float C, float 
         // Delta > 0 here (certified, or FP64 said so): as in the packed path
         const float sq = Dl > 0.0f ? __fmul_rn(Dl, rsqrt_fast(Dl)) : 0.0f;
         const float S = cbrt_fast(__fadd_rn(R, R >= 0.0f ? sq : -sq));
-        const float ST = S != 0.0f ? __fmaf_rn(-Q, rcp_fast(S), S) : 0.0f; // S + T
-        const float x = newton_polish32(A, B, C, D, __fsub_rn(ST, b3));
+        const float T = S != 0.0f ? __fmul_rn(-Q, rcp_fast(S)) : 0.0f;
+        const float x = newton_polish32(A, B, C, D, __fsub_rn(__fadd_rn(S, T), b3));
         if (!isfinite(x)) return quartic_min_fallback64(A, B, C, D, lo, hi, paper_mode);
         return clampf(x, lo, hi);
     }

@@ -121,8 +121,9 @@ SingleShape single_shape(int precision, int m, int q, int64_t rs, int nsm, size_
         }
     }
     // Contiguous equal column chunks over as many SMs as there are warps of
-    // work (FP64 throughput per SM is the scarce resource), one CTA per SM
-    // while that covers every column vector in a single pass, two otherwise.
+    // work (FP64 throughput per SM is the scarce resource), one CTA per SM;
+    // mixed: the wide variant where 256 threads per SM would take more than one
+    // pass (see NT at single_kernel).
     sh.wide = (mixed && ncols > (int64_t)nsm * single_threads(precision, 1) * unit) ? 2 : 1;
     int per_sm = single_blocks_per_sm(precision, m, sh.wide, smem);
     if (per_sm < 1 && sh.wide == 2) {
