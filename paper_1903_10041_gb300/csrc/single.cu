@@ -107,7 +107,10 @@ SingleShape single_shape(int precision, int m, int q, int64_t rs, int nsm, size_
     // cycles anyway) and the cluster barrier and distributed shared memory save
     // the grid barrier and the records' way through L2.  Up to 8 CTAs, the
     // portable cluster size; beyond that a CTA would need several rounds.
-    // n = 100, m = 2, q = 1 FP64: 6.5 -> 5.3 us per iteration.
+    // us per iteration on the grid -> as a cluster, at one CTA and at eight: FP64,
+    // m = 2: n = 100 9.5 -> 7.2, n = 1000 9.5 -> 7.4; m = 4, n = 1000 12.9 -> 11.4;
+    // mixed: n = 100, m = 2 6.0 -> 4.5, n = 4000, m = 4 7.6 -> 6.5 (short solves,
+    // the call's own time included).
     {
         const int64_t cap = mixed ? (int64_t)kBlock * unit : kBlockF64Cluster;
         const int64_t p = (rs + cap - 1) / cap;
