@@ -91,7 +91,7 @@ NCU_TRAFFIC = {
     ("phev n=1000 q=50", "fp64"): {"bytes_per_iter": (7196672 + 60160) / 3330, "src": "457c39ff1bdae819"},
     ("plain n=1e5 m=4 q=20", "mixed"): {"bytes_per_iter": (545884681728 + 173432479744) / 2720, "src": "457c39ff1bdae819"},
 }
-NCU_TRAFFIC_BATCH = {"bytes_per_element_iter": (1811961266176 + 614259118080) / 76330081250.0, "src": "58bddc1cb77dc15c"}
+NCU_TRAFFIC_BATCH = {"bytes_per_element_iter": (1824847392768 + 617704844800) / 76364664590.0, "src": "58ea3e62cb52c56a"}
 # FP64 pipe utilisation (sm__pipe_fp64_cycles_active, % of peak over the active cycles) of the FP64 solve
 # kernel on the PHEV instance, from an ncu capture of the same build: the counted-flop fraction leaves out
 # the Newton steps of the FP32-seeded roots, conversions, comparisons and the per-pair scalar phase.
