@@ -215,6 +215,7 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
         const bool cold = ipar[2] != 0;
         const float mu_div = fpar[3];
         const float rho1 = fpar[0], rho3 = fpar[1], rho4 = fpar[2], iq = fpar[4];
+        const bool tiny_c = tiny_rho3(rho3);
         // lane maxima and minima that only check iterations use: with the staged
         // (m <= 4) update they live in the thread's own shared-memory slots (11
         // floats apart, no bank conflicts) instead of registers across the loop
@@ -245,7 +246,7 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
             }
             double *rec = recs + (size_t)(j + gw) * m * 4;
             // PLAIN: not a check iteration, not cold, no pending mu divisor (nine iterations in
-            // ten), with those branches and their registers compiled out of the loop (not for M = 8,
+            // ten), a normal rho_3, with those branches and their registers compiled out of the loop (not for M = 8,
             // where two copies spill more than the branches cost)
             auto columns = [&](auto plain) {
                 constexpr bool PLAIN = decltype(plain)::value;
@@ -258,7 +259,7 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
                     roll_prologue<M>(ea, j, v * VW, v < v1, stw);
                     for (; v < v1; v += 32) {
                         const int kn = v + 32 < v1 ? (v + 32) * VW : -1;
-                        vec32<M, VW, false, STAGE_ROLL>(ea, uoff, x1nu, j, v * VW, chk, cld, mud, rho1, rho3,
+                        vec32<M, VW, false, STAGE_ROLL>(ea, uoff, x1nu, j, v * VW, chk, cld, PLAIN, mud, rho1, rho3,
                                                         rho4, iq, ghi, glo, fmx, fmn, fcr, fcs, esc, rec + 3, 4, stw, kn);
                     }
                     cp_async_wait0();
@@ -276,19 +277,19 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
                         }
                         cp_async_commit();
                         cp_async_wait1(); // this round's copies have landed
-                        vec32<M, VW, false, STAGE_DOUBLE>(ea, uoff, x1nu, j, v * VW, chk, cld, mud, rho1, rho3,
+                        vec32<M, VW, false, STAGE_DOUBLE>(ea, uoff, x1nu, j, v * VW, chk, cld, PLAIN, mud, rho1, rho3,
                                                           rho4, iq, ghi, glo, fmx, fmn, fcr, fcs, esc, rec + 3, 4, cur);
                     }
                     cp_async_wait0();
                 } else {
                     for (; v < v1; v += 32) {
                         if (v + 32 < v1) prefetch_vec32<M>(ea, j, (v + 32) * VW, cld);
-                        vec32<M, VW, false>(ea, uoff, x1nu, j, v * VW, chk, cld, mud, rho1, rho3, rho4, iq, ghi,
+                        vec32<M, VW, false>(ea, uoff, x1nu, j, v * VW, chk, cld, PLAIN, mud, rho1, rho3, rho4, iq, ghi,
                                             glo, fmx, fmn, fcr, fcs, esc, rec + 3, 4);
                     }
                 }
             };
-            if (M > 4 || check || cold || mu_div != 1.0f) columns(std::false_type{});
+            if (M > 4 || check || cold || mu_div != 1.0f || tiny_c) columns(std::false_type{});
             else columns(std::true_type{});
             {
                 // the piece's sums of all sources at once (warp_many), written by one lane per source

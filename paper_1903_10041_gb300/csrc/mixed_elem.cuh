@@ -290,15 +290,16 @@ __device__ __forceinline__ void st2(float *p, float2 v) { *(float2 *)p = v; }
 // STAGE_ROLL: the inputs come from the lane's rolling stage stg, and each slot
 // group is refilled with the pair k0n (if >= 0) as soon as it is read.  The
 // first column is always < n; the second may be padding (k0 + 1 = n), and
-// then takes no part in the sums and residuals.
+// then takes no part in the sums and residuals.  plain: rho_3 is a normal number
+// (the caller's loop without checks).
 // Where vec32 reads its inputs: global memory, the double stage of
 // stage_vec32 (coefficients and y), or the rolling stage (everything).
 enum { STAGE_NONE = 0, STAGE_DOUBLE = 1, STAGE_ROLL = 2 };
 
 template <int M, int VW, bool C64, int STAGE = STAGE_NONE, class EA>
 __device__ __forceinline__ void vec32(const EA &a, const float *uoff, const float *x1nu,
-                                      int j, int k0, bool check, bool cold, float mu_div, float rho1, float rho3,
-                                      float rho4, float iq, float2 *ghi, float2 *glo, float *dmx, float *dmn,
+                                      int j, int k0, bool check, bool cold, bool plain, float mu_div, float rho1,
+                                      float rho3, float rho4, float iq, float2 *ghi, float2 *glo, float *dmx, float *dmn,
                                       float &cm_r, float &cm_s, unsigned &esc, double *rec, int rstep,
                                       float2 *stg = nullptr, int k0n = -1)
 {
@@ -370,7 +371,7 @@ __device__ __forceinline__ void vec32(const EA &a, const float *uoff, const floa
                 xn = make_float2(quartic_min_fp64cubic(A.x, B.x, C.x, D.x, L.x, H.x, a.xmin_mode),
                                  quartic_min_fp64cubic(A.y, B.y, C.y, D.y, L.y, H.y, a.xmin_mode));
             else
-                xn = quartic_min32x2(A, B, C, D, L, H, a.xmin_mode, esc);
+                xn = quartic_min32x2(A, B, C, D, L, H, a.xmin_mode, esc, !plain);
             if (!jac) xsum = add2(xsum, sub2(xn, x0));
             sx = ff2_addf(sx, xn); // sum_i x of (e), (f) in source order
             if (check) dx = ff2_add(dx, ff2_two_sum(xn, neg2(x0)));

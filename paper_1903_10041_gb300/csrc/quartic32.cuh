@@ -32,14 +32,18 @@ namespace admm_impl {
 // few-ulp errors are removed by the Newton step that follows (the root it
 // converges to depends only on the coefficients), and the discriminant bound
 // below allows for a reciprocal that is off by 2 ulp.  A denormal operand
-// gives an infinity or a zero, and with it a non-finite root or an
-// uncertified discriminant, which the callers send to FP64.
+// gives an infinity and one above 2^126 a zero.  Where a root is such a
+// quotient itself (A = 0) or A's reciprocal left the range, the scalar code
+// takes FP64 (rcp_in_range); elsewhere an infinity ends in a non-finite root or
+// an uncertified discriminant, which go to FP64 too.
 __device__ __forceinline__ float rcp_fast(float v)
 {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
     return r;
 }
+// Is r = rcp_fast(v) the reciprocal of a v > 0 (not flushed to an infinity or a zero)?
+__device__ __forceinline__ bool rcp_in_range(float r) { return __float_as_uint(r) - 1u < 0x7f7fffffu; }
 __device__ __forceinline__ float rsqrt_fast(float v)
 {
     float r;
@@ -142,7 +146,11 @@ static __device__ __noinline__ int cubic_branch64(float A, float B, float C, flo
 __device__ __forceinline__ float quartic_min32(float A, float B, float C, float D, float lo, float hi,
                                                int paper_mode, unsigned &esc)
 {
-    if (A == 0.0f) return clampf(__fmul_rn(-D, rcp_fast(__fadd_rn(C, C))), lo, hi);
+    if (A == 0.0f) {
+        const float r = rcp_fast(__fadd_rn(C, C));
+        if (!rcp_in_range(r)) return quartic_min_fallback64(A, B, C, D, lo, hi, paper_mode);
+        return clampf(__fmul_rn(-D, r), lo, hi);
+    }
     // unfused, so that an input near a double root or a tie keeps the rounding it always had
     const float inv = rcp_fast(A);
     const float b = __fmul_rn(__fmul_rn(0.75f, B), inv);
@@ -167,8 +175,9 @@ __device__ __forceinline__ float quartic_min32(float A, float B, float C, float 
     int branch; // 0 Cardano, 1 triple, 2 trig
     if (Dl > bound) branch = 0;
     else if (Dl < -bound) branch = 2;
-    else {
+    else { // among them every A whose reciprocal left the range: Delta is 0 or NaN, or the bound infinite
         ++esc;
+        if (!rcp_in_range(inv)) return quartic_min_fallback64(A, B, C, D, lo, hi, paper_mode);
         branch = cubic_branch64(A, B, C, D);
     }
     if (branch == 1) return clampf(-b3, lo, hi);
@@ -591,8 +600,12 @@ static __device__ __noinline__ float2 quartic_min32_lanes(float2 A, float2 B, fl
     return x;
 }
 
+// In step (a) 2 C is at least rho_3 where A = 0, so a test of rho_3 says whether it may be denormal.
+__device__ __forceinline__ bool tiny_rho3(float rho3) { return rho3 < 1.17549435e-38f; }
+
+// tiny_c: 2 C may be denormal where A = 0, so look for an infinite reciprocal.
 __device__ __forceinline__ float2 quartic_min32x2(float2 A, float2 B, float2 C, float2 D, float2 lo, float2 hi,
-                                                  int paper_mode, unsigned &esc)
+                                                  int paper_mode, unsigned &esc, bool tiny_c)
 {
 #ifndef ADMM_COMPENSATED_POLISH
     if (A.x > 0.0f && A.y > 0.0f) {
@@ -626,8 +639,9 @@ __device__ __forceinline__ float2 quartic_min32x2(float2 A, float2 B, float2 C, 
     }
     if (A.x == 0.0f && A.y == 0.0f) { // quadratic on both lanes
         const float2 C2 = add2(C, C);
-        const float2 x = mul2(neg2(D), make_float2(rcp_fast(C2.x), rcp_fast(C2.y)));
-        return make_float2(clampf(x.x, lo.x, hi.x), clampf(x.y, lo.y, hi.y));
+        const float2 r = make_float2(rcp_fast(C2.x), rcp_fast(C2.y)), x = mul2(neg2(D), r);
+        if (!tiny_c || r.x * r.y < INFINITY) // (two finite ones whose product is not: the same bits lane by lane)
+            return make_float2(clampf(x.x, lo.x, hi.x), clampf(x.y, lo.y, hi.y));
     }
 #endif
     return quartic_min32_lanes(A, B, C, D, lo, hi, paper_mode, &esc);

@@ -614,8 +614,9 @@ __global__ void __launch_bounds__(NT, 1) single_kernel(SingleArgs a)
                                     a.xmin_mode,         a.cq,                a.cj,
                                     a.dbg};
                 const int kn = min(ke, n); // padding columns k >= n are skipped
+                const bool tiny_c = tiny_rho3(rho3);
                 // PLAIN: not a check iteration, not cold, no pending mu divisor (nine iterations in
-                // ten), with those branches and their registers compiled out of the loop (n = 1e5,
+                // ten), a normal rho_3, with those branches and their registers compiled out of the loop (n = 1e5,
                 // m = 4, q = 20: 91.3 -> 80.2 us per iteration).  Not for M = 8, where two copies
                 // spill more than the branches cost (m = 6: 23.0 -> 25.9).
                 auto columns = [&](auto plain) {
@@ -632,7 +633,7 @@ __global__ void __launch_bounds__(NT, 1) single_kernel(SingleArgs a)
                         for (int k0 = k00; k0 < kn; k0 += stride * VW) {
                             const int k0n = k0 + stride * VW < kn ? k0 + stride * VW : -1;
                             vec32<M, VW, PREC == ADMM_MIXED_FP64CUBIC, STAGE_ROLL>(
-                                ea, sm.uoff, sm.x1nu, j, k0, chk, cld, mud, rho1, rho3, rho4, iq, ghi, glo,
+                                ea, sm.uoff, sm.x1nu, j, k0, chk, cld, PLAIN, mud, rho1, rho3, rho4, iq, ghi, glo,
                                 fmx, fmn, fcr, fcs, esc, rec, rstep, stw, k0n);
                         }
                         cp_async_wait0();
@@ -641,12 +642,12 @@ __global__ void __launch_bounds__(NT, 1) single_kernel(SingleArgs a)
                             if constexpr (NT > kBlock) // several vectors per thread: fetch the next one into L2
                                 if (k0 + stride * VW < kn) prefetch_vec32<M>(ea, j, k0 + stride * VW, cld);
                             vec32<M, VW, PREC == ADMM_MIXED_FP64CUBIC>(ea, sm.uoff, sm.x1nu, j, k0, chk, cld,
-                                                                       mud, rho1, rho3, rho4, iq, ghi, glo,
+                                                                       PLAIN, mud, rho1, rho3, rho4, iq, ghi, glo,
                                                                        fmx, fmn, fcr, fcs, esc, rec, rstep);
                         }
                     }
                 };
-                if (M > 4 || check || cold || mudf != 1.0f) columns(std::false_type{});
+                if (M > 4 || check || cold || mudf != 1.0f || tiny_c) columns(std::false_type{});
                 else columns(std::true_type{});
                 flush_segments32<M, NWP, CL>(a, par, jb, ns, ghi, glo, fmx, fmn, fcr, fcs, check, m, sp, sm);
             }
