@@ -302,7 +302,7 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
                 const FF v = warp_many<M>(g, add);
                 const int i = slot_of<M>(lane);
                 const bool out_lane = lane % (32 / M) == 0 && i < m;
-                if (out_lane) rec[i * 4 + 0] = f32_to_f64_int(v.hi) + f32_to_f64_int(v.lo);
+                if (out_lane) rec[i * 4 + 0] = f32_to_f64_nan(v.hi) + f32_to_f64_nan(v.lo);
                 if (check) {
                     auto mx = [](float k, float u, int o) { return fmaxf(k, __shfl_xor_sync(0xffffffffu, u, o)); };
                     auto mn = [](float k, float u, int o) { return fminf(k, __shfl_xor_sync(0xffffffffu, u, o)); };
@@ -311,17 +311,17 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
                     for (int t = 0; t < M; ++t) th[t] = fmx[t], tl[t] = fmn[t];
                     const float hi = warp_many<M>(th, mx), lo = warp_many<M>(tl, mn);
                     if (out_lane) {
-                        rec[i * 4 + 1] = f32_to_f64_int(hi);
-                        rec[i * 4 + 2] = f32_to_f64_int(lo);
+                        rec[i * 4 + 1] = f32_to_f64_nan(hi);
+                        rec[i * 4 + 2] = f32_to_f64_nan(lo);
                     }
                 }
             }
         }
         if (check) {
-            const float wr = warp_max(fcr), ws = warp_max(fcs);
+            const float wr = warp_max_nonneg(fcr), ws = warp_max_nonneg(fcs);
             if (lane == 0) {
-                cmax[(par * NWT + wl) * 2 + 0] = f32_to_f64_int(wr);
-                cmax[(par * NWT + wl) * 2 + 1] = f32_to_f64_int(ws);
+                cmax[(par * NWT + wl) * 2 + 0] = f32_to_f64_nan(wr);
+                cmax[(par * NWT + wl) * 2 + 1] = f32_to_f64_nan(ws);
             }
         }
         sync_team(); // every record of this iteration is complete and visible
@@ -347,7 +347,7 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
                 const int w = rows[j] & 0xffff; // k = 0 lies in the first warp's piece
                 const double *rb = recs;
                 if constexpr (KIND == TEAM_CLUSTER) rb = cg::this_cluster().map_shared_rank(recs, w / NWT);
-                const double x0 = f32_to_f64_int(*(const float *)(rb + ((size_t)(j + w) * m + i) * 4 + 3));
+                const double x0 = f32_to_f64_nan(*(const float *)(rb + ((size_t)(j + w) * m + i) * 4 + 3));
                 const double d = x0 - nu[i * q + j];
                 x0s[i * q + j] = x0;
                 sum = j == lane ? d : sum + d;
@@ -357,7 +357,7 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
                 const int pr = i * q + j;
                 const double d = xn - x0s[pr], nun = nu[pr] + d;      // (h)
                 nu[pr] = nun;
-                x1nu[pr] = f64_to_f32_int(xn + nun);
+                x1nu[pr] = f64_to_f32_nan(xn + nun);
                 if (check) r4m = max_nonneg(r4m, fabs(d));
             }
             if (lane == 0) x1[i] = xn;
@@ -410,7 +410,7 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
                 zeta[pr] = zn;
                 hh[pr] = hn;
                 pp[pr] = pv + e;                                      // (i)
-                uoff[pr] = f64_to_f32_int(zn + lamn);
+                uoff[pr] = f64_to_f32_nan(zn + lamn);
             }
         }
         if (check) { // per-warp maxima of the residual terms

@@ -104,10 +104,20 @@ template <class T> __device__ __forceinline__ T warp_max(T v)
 // Maxima of non-negative doubles (residual terms, absolute values): for
 // x, y >= 0 the order of their IEEE-754 bit patterns read as signed 64-bit
 // integers is the order of the values, so these run on the integer pipes
-// instead of the FP64 pipe (1/64 of the FP32 rate on this GPU).
+// instead of the FP64 pipe (1/64 of the FP32 rate on this GPU).  A NaN without
+// its sign ranks above infinity, so it is kept and fails the stop test; the FP32
+// forms are there for that alone.
 __device__ __forceinline__ double max_nonneg(double a, double b)
 {
     return __longlong_as_double(max(__double_as_longlong(a), __double_as_longlong(b)));
+}
+__device__ __forceinline__ float max_nonneg(float a, float b)
+{
+    return __uint_as_float(max(__float_as_uint(a), __float_as_uint(b)));
+}
+__device__ __forceinline__ float warp_max_nonneg(float v)
+{
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
 }
 __device__ __forceinline__ double warp_max_nonneg(double v)
 {

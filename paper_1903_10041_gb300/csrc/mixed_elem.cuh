@@ -407,13 +407,14 @@ __device__ __forceinline__ void vec32(const EA &a, const float *uoff, const floa
     const FF2 mnew = {make_float2(v.hi.x < 0.0f ? nv.hi.x : 0.0f, v.hi.y < 0.0f ? nv.hi.y : 0.0f),
                       make_float2(v.hi.x < 0.0f ? nv.lo.x : 0.0f, v.hi.y < 0.0f ? nv.lo.y : 0.0f)}; // (f)
     if (check) {
-        const FF2 t = ff2_add(mnew, ff2_neg(muf)); // s - sum_i x + y
+        // s - sum_i x + y; a column whose v left the FP32 range has s = mu = 0 and no residual: NaN
+        const FF2 t = ff2_add(mnew, ff2_neg(muf));
         const FF2 d = ff2_add(ff2_add(sv, ff2_neg(stf)), ff2_neg(dx)); // s - s~ - sum_i (x - x~)
-        cm_r = fmaxf(cm_r, fabsf(t.hi.x + t.lo.x));
-        cm_s = fmaxf(cm_s, fabsf(d.hi.x + d.lo.x));
+        cm_r = max_nonneg(cm_r, fabsf(fmaf(v.hi.x, 0.0f, t.hi.x + t.lo.x)));
+        cm_s = max_nonneg(cm_s, fabsf(d.hi.x + d.lo.x));
         if (v1) {
-            cm_r = fmaxf(cm_r, fabsf(t.hi.y + t.lo.y));
-            cm_s = fmaxf(cm_s, fabsf(d.hi.y + d.lo.y));
+            cm_r = max_nonneg(cm_r, fabsf(fmaf(v.hi.y, 0.0f, t.hi.y + t.lo.y)));
+            cm_s = max_nonneg(cm_s, fabsf(d.hi.y + d.lo.y));
         }
     }
     st2(a.s + col, sv.hi);

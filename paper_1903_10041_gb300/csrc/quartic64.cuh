@@ -55,12 +55,26 @@ __device__ __forceinline__ float f64_to_f32_int(double v)
     const unsigned r = ah < (897u << 20) ? 0u : (ah >= (1151u << 20) ? 0x7f800000u : f);
     return __uint_as_float(r | (hi & 0x80000000u));
 }
-// (double)v, exact, for a zero or a normal v (a denormal gives a signed zero).
+// The same with a NaN kept (a quiet one, as arithmetic gives).
+__device__ __forceinline__ float f64_to_f32_nan(double v)
+{
+    const float r = f64_to_f32_int(v);
+    return (__double2hiint(v) & 0x7ff80000) == 0x7ff80000 ? NAN : r;
+}
+// (double)v, exact, for a zero or a normal v (a denormal gives a signed zero; no infinities, no NaN).
 __device__ __forceinline__ double f32_to_f64_int(float v)
 {
     const unsigned b = __float_as_uint(v), a = b & 0x7fffffffu;
     const bool z = a < 0x00800000u;
     return __hiloint2double((int)((b & 0x80000000u) | (z ? 0u : (a >> 3) + (896u << 20))), (int)(z ? 0u : b << 29));
+}
+// The same with infinities and NaN kept: what a solve's sums and residuals go through.
+__device__ __forceinline__ double f32_to_f64_nan(float v)
+{
+    const unsigned b = __float_as_uint(v), a = b & 0x7fffffffu;
+    const bool z = a < 0x00800000u;
+    const unsigned e = a < 0x7f800000u ? 896u << 20 : 1792u << 20; // exponent 255 becomes 2047
+    return __hiloint2double((int)((b & 0x80000000u) | (z ? 0u : (a >> 3) + e)), (int)(z ? 0u : b << 29));
 }
 // (float)v truncated, half the instructions: for seeds, whose error bounds
 // count two units of 2^-24 per converted value.  Magnitudes outside the FP32

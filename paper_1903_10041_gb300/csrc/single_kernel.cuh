@@ -443,15 +443,15 @@ __device__ __forceinline__ void flush_segments32(const SingleArgs &a, int par, i
     }
     if (check) {
         const float hi = warp_many<M>(fmx, mx), lo = warp_many<M>(fmn, mn);
-        cm_r = warp_max(cm_r);
-        cm_s = warp_max(cm_s);
+        cm_r = warp_max_nonneg(cm_r);
+        cm_s = warp_max_nonneg(cm_s);
         if (lane % (32 / M) == 0) {
             rw[2] = hi;
             rw[3] = lo;
         }
         if (lane == 0) {
-            sm.mx[w * 8] = f32_to_f64_int(cm_r);
-            sm.mx[w * 8 + 1] = f32_to_f64_int(cm_s);
+            sm.mx[w * 8] = f32_to_f64_nan(cm_r);
+            sm.mx[w * 8 + 1] = f32_to_f64_nan(cm_s);
         }
     }
     if (lane == 0) sm.segof[w] = sp.seg;
@@ -475,8 +475,8 @@ __device__ __forceinline__ void flush_segments32(const SingleArgs &a, int par, i
             }
         }
         if (hl == 0 && t < ns * m) {
-            put_record<CL>(a, sm, par, jb + sg, i, f32_to_f64_int(r.hi) + f32_to_f64_int(r.lo), check,
-                           f32_to_f64_int(hi), f32_to_f64_int(lo));
+            put_record<CL>(a, sm, par, jb + sg, i, f32_to_f64_nan(r.hi) + f32_to_f64_nan(r.lo), check,
+                           f32_to_f64_nan(hi), f32_to_f64_nan(lo));
         }
     }
 }
@@ -697,8 +697,8 @@ __global__ void __launch_bounds__(NT, 1) single_kernel(SingleArgs a)
                 for (int j = lane; j < q; j += 32) {
                     // x at k = 0: FP64 in the FP64 kernel, FP32 in the slot's first four bytes in the mixed ones
                     double x0;
-                    if constexpr (CL) x0 = MIXED ? f32_to_f64_int(*(const float *)remote(j, 0, i, 3)) : *remote(j, 0, i, 3);
-                    else x0 = MIXED ? f32_to_f64_int(__ldcg((const float *)(rr.x0() + i * q + j))) : ldcg(rr.x0() + i * q + j);
+                    if constexpr (CL) x0 = MIXED ? f32_to_f64_nan(*(const float *)remote(j, 0, i, 3)) : *remote(j, 0, i, 3);
+                    else x0 = MIXED ? f32_to_f64_nan(__ldcg((const float *)(rr.x0() + i * q + j))) : ldcg(rr.x0() + i * q + j);
                     const double d = x0 - sm.nu[i * q + j];
                     sm.x0[i * q + j] = x0;
                     sum = j == lane ? d : sum + d;
@@ -708,7 +708,7 @@ __global__ void __launch_bounds__(NT, 1) single_kernel(SingleArgs a)
                     const int pr = i * q + j;
                     const double d = x1n - sm.x0[pr], nun = sm.nu[pr] + d; // (h)
                     sm.nu[pr] = nun;
-                    if (MIXED) sm.x1nu[pr] = f64_to_f32_int(x1n + nun);
+                    if (MIXED) sm.x1nu[pr] = f64_to_f32_nan(x1n + nun);
                     if (check) r4m = max_nonneg(r4m, fabs(d));
                 }
                 if (lane == 0) sm.x1[i] = x1n;
@@ -777,7 +777,7 @@ __global__ void __launch_bounds__(NT, 1) single_kernel(SingleArgs a)
                 sm.zeta[pr] = zn;
                 sm.h[pr] = hn;
                 sm.p[pr] = pp + e;                                    // (i)
-                if (MIXED) sm.uoff[pr] = f64_to_f32_int(zn + lamn);
+                if (MIXED) sm.uoff[pr] = f64_to_f32_nan(zn + lamn);
                 else sm.zl[pr] = zn + lamn;
             }
         }
