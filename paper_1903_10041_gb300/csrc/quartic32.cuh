@@ -518,11 +518,13 @@ __device__ __forceinline__ double elem_min64_seeded(const Elem64 &p, float hr1f,
     return elem_min64(p, lo, hi, paper_mode);
 }
 
-// The same without losses: H(x) = C x + Dh.
+// The same without losses: H(x) = C x + Dh.  A Dh beyond the FP32 range (an
+// infinity or a NaN too, which the seed's conversion makes finite) takes the
+// division and the comparing clamp.
 __device__ __forceinline__ double elem_min64_linear(double C, double Dh, double lo, double hi)
 {
-    const float Cf = f64_to_f32_seed(C), rf = rcp_fast(Cf), xf = -f64_to_f32_seed(Dh) * rf;
-    if (rf >= 1.2e-38f && rf < 1.0e38f && fabsf(xf) < 1.0e30f) {
+    const float Cf = f64_to_f32_seed(C), Df = f64_to_f32_seed(Dh), rf = rcp_fast(Cf), xf = -Df * rf;
+    if (rf >= 1.2e-38f && rf < 1.0e38f && fabsf(xf) < 1.0e30f && fabsf(Df) < 1.0e37f) {
         const double r = f32_to_f64_seed(rf);
         double x = f32_to_f64_seed(xf);
         x = fma(-fma(C, x, Dh), r, x);
