@@ -182,7 +182,7 @@ __device__ __forceinline__ float quartic_min32(float A, float B, float C, float 
     }
     if (branch == 1) return clampf(-b3, lo, hi);
     if (branch == 0) {
-        // Delta > 0 here (certified, or FP64 said so): as in the packed path
+        // Delta > 0 here (certified, or FP64 said so)
         const float sq = Dl > 0.0f ? __fmul_rn(Dl, rsqrt_fast(Dl)) : 0.0f;
         const float S = cbrt_fast(__fadd_rn(R, R >= 0.0f ? sq : -sq));
         const float T = S != 0.0f ? __fmul_rn(-Q, rcp_fast(S)) : 0.0f;
@@ -657,8 +657,9 @@ __device__ __forceinline__ float2 quartic_min32x2(float2 A, float2 B, float2 C, 
 // quartics, 2^26 of them 1014 -> 355 us).  The decisions are those of quartic_min32: the branch outside
 // its error bound, the lower minimum where |br| of F(u) - F(v) = (u - v) br
 // exceeds 2e-5 of the sum of its terms' magnitudes (FP32 errs by a few 1e-7
-// of it).  A pair with anything nearer than that, A = 0, or a value that is
-// not finite goes through quartic_min32_lanes.
+// of it).  okx, oky: a lane with anything nearer than that, A = 0, or a value that
+// is not finite is left to quartic_min32.  Each lane's result depends on its own
+// element alone.
 __device__ __forceinline__ float2 min2(float2 a, float2 b) { return make_float2(fminf(a.x, b.x), fminf(a.y, b.y)); }
 __device__ __forceinline__ float2 max2(float2 a, float2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
 __device__ __forceinline__ float2 sel2(bool px, bool py, float2 a, float2 b)
@@ -677,7 +678,7 @@ __device__ __forceinline__ float2 cos_third2(float2 a)
 }
 
 __device__ __forceinline__ float2 quartic_min32x2_wells(float2 A, float2 B, float2 C, float2 D, float2 lo, float2 hi,
-                                                        int paper_mode, unsigned &esc)
+                                                        int paper_mode, bool &okx, bool &oky)
 {
     const float2 inv = make_float2(rcp_fast(A.x), rcp_fast(A.y));
     const float2 b = mul2(mul2(splat2(0.75f), B), inv);
@@ -696,7 +697,8 @@ __device__ __forceinline__ float2 quartic_min32x2_wells(float2 A, float2 B, floa
     const float2 mR = fma2(abs2(b3), add2(b3s, ahc), ahd);
     const float2 bound = mul2(splat2(7.68e-6f), fma2(Qs, mQ, mul2(abs2(R), mR)));
     const bool cx = Dl.x > bound.x, cy = Dl.y > bound.y, tx = Dl.x < -bound.x, ty = Dl.y < -bound.y;
-    bool ok = A.x > 0.0f && A.y > 0.0f && (cx || tx) && (cy || ty);
+    okx = A.x > 0.0f && (cx || tx);
+    oky = A.y > 0.0f && (cy || ty);
     // sqrt(Delta) on the Cardano branch, sqrt(-Q) on the trig branch
     const float2 rad = sel2(cx, cy, Dl, nQ);
     const float2 rs = make_float2(rsqrt_fast(rad.x), rsqrt_fast(rad.y));
@@ -718,7 +720,8 @@ __device__ __forceinline__ float2 quartic_min32x2_wells(float2 A, float2 B, floa
     }
     u = newton_polish32x2(A, B, C, D, u);
     const float2 fin = fma2(u, splat2(0.0f), mul2(v, splat2(0.0f))); // 0 where u and v are finite, else NaN
-    ok = ok && fin.x + fin.y == 0.0f;
+    okx = okx && fin.x == 0.0f;
+    oky = oky && fin.y == 0.0f;
     float2 x = max2(min2(u, hi), lo);
     if (any_trig) {
         const float2 vc = max2(min2(v, hi), lo);
@@ -731,10 +734,10 @@ __device__ __forceinline__ float2 quartic_min32x2_wells(float2 A, float2 B, floa
         const float2 mb = add2(fma2(q4, as, abs2(b3q)), fma2(ahc, as, add2(ahd, ahd)));
         const float2 lim = mul2(splat2(2.0e-5f), mb);
         const bool nx = tx && p.x != r.x, ny = ty && p.y != r.y; // u < v: the larger root where br < 0
-        ok = ok && (!nx || fabsf(br.x) > lim.x) && (!ny || fabsf(br.y) > lim.y);
+        okx = okx && (!nx || fabsf(br.x) > lim.x);
+        oky = oky && (!ny || fabsf(br.y) > lim.y);
         x = sel2(nx && br.x < 0.0f, ny && br.y < 0.0f, vc, x);
     }
-    if (!ok) return quartic_min32_lanes(A, B, C, D, lo, hi, paper_mode, &esc);
     return x;
 }
 

@@ -62,16 +62,42 @@ __global__ void __launch_bounds__(256) quartic_many_f64(const double *A, const d
     report_bad(nbad, bad);
 }
 
-// A pair with A = 0 or an invalid element, out of line.
-__device__ __noinline__ float2 quartic_pair_rest(float2 a, float2 b, float2 c, float2 d, float2 l, float2 h, int mode,
-                                                 int *nbad)
+// The lanes that the packed code left (a NaN in r): solved alone, or counted as invalid.  Out of line.
+__device__ __noinline__ float2 quartic_pair_rest(float2 a, float2 b, float2 c, float2 d, float2 l, float2 h, float2 r,
+                                                 int mode, int *nbad)
 {
     unsigned esc = 0;
-    const bool okx = quartic_ok(a.x, b.x, c.x, d.x, l.x, h.x), oky = quartic_ok(a.y, b.y, c.y, d.y, l.y, h.y);
-    if (okx && oky) return quartic_min32_lanes(a, b, c, d, l, h, mode, &esc);
-    *nbad += (okx ? 0 : 1) + (oky ? 0 : 1);
-    return make_float2(okx ? quartic_min32(a.x, b.x, c.x, d.x, l.x, h.x, mode, esc) : NAN,
-                       oky ? quartic_min32(a.y, b.y, c.y, d.y, l.y, h.y, mode, esc) : NAN);
+    if (isnan(r.x)) {
+        if (quartic_ok(a.x, b.x, c.x, d.x, l.x, h.x)) r.x = quartic_min32(a.x, b.x, c.x, d.x, l.x, h.x, mode, esc);
+        else ++*nbad;
+    }
+    if (isnan(r.y)) {
+        if (quartic_ok(a.y, b.y, c.y, d.y, l.y, h.y)) r.y = quartic_min32(a.y, b.y, c.y, d.y, l.y, h.y, mode, esc);
+        else ++*nbad;
+    }
+    return r;
+}
+
+// One pair; an element's bits depend on its own data alone.
+__device__ __forceinline__ float2 quartic_pair(float2 a, float2 b, float2 c, float2 d, float2 l, float2 h, int mode,
+                                               int *nbad)
+{
+    // finite coefficients (their magnitudes' sum is) and lo <= hi; anything else is looked at lane by lane
+    const float2 m = add2(add2(abs2(a), abs2(b)), add2(abs2(c), abs2(d)));
+    bool okx, oky;
+    const float2 r = quartic_min32x2_wells(a, b, c, d, l, h, mode, okx, oky);
+    okx = okx && m.x < INFINITY && l.x <= h.x;
+    oky = oky && m.y < INFINITY && l.y <= h.y;
+    if (okx && oky) return r;
+    return quartic_pair_rest(a, b, c, d, l, h, make_float2(okx ? r.x : NAN, oky ? r.y : NAN), mode, nbad);
+}
+
+// The last element of an odd count, paired with x^4 + x^2.  Out of line.
+__device__ __noinline__ float quartic_odd(float a, float b, float c, float d, float l, float h, int mode, int *nbad)
+{
+    return quartic_pair(make_float2(a, 1.0f), make_float2(b, 0.0f), make_float2(c, 1.0f), make_float2(d, 0.0f),
+                        make_float2(l, -1.0f), make_float2(h, 1.0f), mode, nbad)
+        .x;
 }
 
 constexpr int kThreads32 = 128, kPerSm = 64;
@@ -80,7 +106,6 @@ __global__ void __launch_bounds__(kThreads32, 8) quartic_many_f32(const float *A
                                                         int64_t count, int mode, float *x, int *bad)
 {
     const int64_t pairs = count / 2;
-    unsigned esc = 0;
     int nbad = 0;
     const int64_t step = (int64_t)gridDim.x * blockDim.x;
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -97,23 +122,11 @@ __global__ void __launch_bounds__(kThreads32, 8) quartic_many_f32(const float *A
     for (; t < pairs; t += step) {
         const float2 a = na, b = nb, c = nc, d = nd, l = nl, h = nh;
         if (t + step < pairs) load(t + step);
-        // finite coefficients (their magnitudes' sum is), A > 0, lo <= hi; anything else is looked at lane by lane
-        const float2 m = add2(add2(abs2(a), abs2(b)), add2(abs2(c), abs2(d)));
-        float2 r;
-        if (m.x < INFINITY && m.y < INFINITY && a.x > 0.0f && a.y > 0.0f && l.x <= h.x && l.y <= h.y)
-            r = quartic_min32x2_wells(a, b, c, d, l, h, mode, esc);
-        else
-            r = quartic_pair_rest(a, b, c, d, l, h, mode, &nbad);
-        ((float2 *)x)[t] = r;
+        ((float2 *)x)[t] = quartic_pair(a, b, c, d, l, h, mode, &nbad);
     }
     if (count % 2 == 1 && blockIdx.x == 0 && threadIdx.x == 0) {
-        const int64_t t = count - 1; // the odd element
-        if (quartic_ok(A[t], B[t], C[t], D[t], lo[t], hi[t])) {
-            x[t] = quartic_min32(A[t], B[t], C[t], D[t], lo[t], hi[t], mode, esc);
-        } else {
-            x[t] = NAN;
-            ++nbad;
-        }
+        const int64_t u = count - 1; // the odd element
+        x[u] = quartic_odd(A[u], B[u], C[u], D[u], lo[u], hi[u], mode, &nbad);
     }
     report_bad(nbad, bad);
 }
