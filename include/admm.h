@@ -224,9 +224,13 @@ admm_status admm_selftest_bounds(int *status_out, long long *index_out);
  * Pi(argmin)).  Arrays are [count], host memory (on_device = 0: copied to
  * and from the device inside the call, the paper's timing with copies) or
  * device memory (on_device = 1, checked: other pointers give ADMM_EINVAL);
- * the caller owns them.  admm_quartic_min
- * uses the solver's FP64 minimiser; admm_quartic_min_f32 the mixed
- * solver's FP32 one (device arrays 8-byte aligned).  Runs on `stream` and
+ * the caller owns them (FP32 device arrays 8-byte aligned).  Both run
+ * variants of the solver's minimisers made for many quartics of every
+ * branch: the same Algorithm 1 with the branch decided as FP64 decides it,
+ * but not the solver's code, so neither their bits nor their times are the
+ * solver's.  admm_quartic_min finds the root in FP32 where that is certain
+ * and refines it in FP64; admm_quartic_min_f32 works on pairs in FP32.
+ * x[t] depends on element t alone.  Runs on `stream` and
  * returns after it has finished.  Each element needs A >= 0, C > 0 when
  * A = 0, lo <= hi and finite coefficients; any other element gets x = NaN
  * and the call returns ADMM_EINVAL (the others are still solved).
