@@ -12,6 +12,8 @@
 #include <thread>
 #include <vector>
 
+#include <cuda.h>
+
 #include "store.h"
 #include "trace.h"
 
@@ -115,7 +117,8 @@ struct admm_batch {
     int *d_q = nullptr;     // three queue heads
     double *d_out = nullptr, *h_out = nullptr;
     double *d_tmp = nullptr;
-    BatchExport *d_export = nullptr; // [count], admm_batch_wait
+    BatchExport *d_export = nullptr;  // [count], admm_batch_wait
+    std::vector<BatchExport> exports; // what it copies there; room for count from the start
     int nX = 0, nL = 0, nS = 0, cluster = 1;
     size_t slice = 0, smem = 0;
     int stage_off = 0;       // byte offset of the coefficient stages in a CTA's shared memory
@@ -298,14 +301,45 @@ __global__ void batch_export_kernel(const BatchInst *inst, const BatchExport *ex
         for (int i = threadIdx.x; i < I.m; i += blockDim.x) e.x1[i] = scal[I.off_scal + 5 * mq + i];
 }
 
-// May the export kernel write n doubles at p?  (Memory of this device, or managed.)
-bool writable_here(const admm_batch *b, const double *p)
+// Allocation that holds device pointer p, by the driver (loaded by the runtime already).
+bool allocation_of(const void *p, uintptr_t &base, size_t &size)
 {
-    if (!p) return true;
-    cudaPointerAttributes at{};
-    if (((uintptr_t)p & 7) != 0 || cudaPointerGetAttributes(&at, p) != cudaSuccess) return cudaGetLastError(), false;
-    return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == b->dev);
+    using Fn = CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const Fn fn = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult r{};
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+            r != cudaDriverEntryPointSuccess)
+            return cudaGetLastError(), (Fn) nullptr;
+        return (Fn)f;
+    }();
+    CUdeviceptr at = 0;
+    if (!fn || fn(&at, &size, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return false;
+    base = (uintptr_t)at;
+    return true;
 }
+
+// Which result buffers the export kernel may write: 8-byte aligned memory of
+// this device, or managed, that the allocation holds to its last byte.  Keeps
+// the last allocation found for the length of one call: the buffers of many
+// instances are usually ranges of one.
+struct ExportTarget {
+    int dev;
+    uintptr_t base = 0;
+    size_t size = 0;
+
+    bool holds(const double *p, size_t n)
+    {
+        if (!p) return true;
+        if (((uintptr_t)p & 7) != 0) return false;
+        if (range_holds(base, size, (uintptr_t)p, 8 * n)) return true;
+        cudaPointerAttributes at{};
+        if (cudaPointerGetAttributes(&at, p) != cudaSuccess) return cudaGetLastError(), false;
+        if (at.type != cudaMemoryTypeManaged && !(at.type == cudaMemoryTypeDevice && at.device == dev)) return false;
+        if (!allocation_of(p, base, size)) return base = size = 0, false;
+        return range_holds(base, size, (uintptr_t)p, 8 * n);
+    }
+};
 
 } // namespace
 
@@ -322,6 +356,7 @@ admm_status admm_batch_create(const admm_problem *probs, int32_t count, const ad
     if (!batch_params_ok(prm, why)) return bfail(prm && prm->precision != ADMM_MIXED ? ADMM_EUNSUPPORTED : ADMM_EINVAL, why);
     admm_batch *b = new admm_batch();
     b->count = count;
+    b->exports.reserve(count);
     b->prm = *prm;
     auto bail = [&](admm_status s) {
         batch_free(b);
@@ -482,7 +517,9 @@ admm_status admm_batch_wait(admm_batch *b, void *stream, admm_result *results)
         return bfail(ADMM_EBOUNDS, "element access out of bounds: array " + std::to_string((int)(rec >> 56) - 1) +
                                        ", index " + std::to_string((long long)(rec & 0x00FFFFFFFFFFFFFFull)));
     admm_status worst = ADMM_OK;
-    std::vector<BatchExport> direct;
+    std::vector<BatchExport> &direct = b->exports;
+    direct.clear();
+    ExportTarget target{b->dev};
     for (int t = 0; t < b->count; ++t) {
         const double *o = b->h_out + (size_t)t * kInfo;
         admm_status s = o[12] != 0.0 ? (admm_status)(int)o[12] : (o[1] != 0.0 ? ADMM_OK : ADMM_ENOTCONVERGED);
@@ -496,7 +533,8 @@ admm_status admm_batch_wait(admm_batch *b, void *stream, admm_result *results)
         r.objective = o[11];
         r.status = s;
         if (!r.x && !r.x1) continue;
-        if (r.on_device && writable_here(b, r.x) && writable_here(b, r.x1)) {
+        const BatchInst &I = b->inst[t];
+        if (r.on_device && target.holds(r.x, (size_t)I.m * I.q * I.n) && target.holds(r.x1, I.m)) {
             direct.push_back({r.x, r.x1, t});
             continue;
         }
@@ -504,7 +542,7 @@ admm_status admm_batch_wait(admm_batch *b, void *stream, admm_result *results)
         st_out.x = r.x;
         st_out.x1 = r.x1;
         st_out.on_device = r.on_device;
-        BTRY(store_get_state(b->store, b->inst[t], &st_out, b->d_tmp, st));
+        BTRY(store_get_state(b->store, I, &st_out, b->d_tmp, st));
     }
     // x of every instance with device buffers in one launch (one by one, with two copies and two
     // synchronisations each, 600 instances took 19 ms and 4096 about 100 ms)

@@ -26,6 +26,12 @@ class RangeAlloc {
     std::map<int64_t, int64_t> free_; // start -> length
 };
 
+// Do the bytes [p, p + bytes) lie in the allocation [base, base + size)?
+inline bool range_holds(uintptr_t base, size_t size, uintptr_t p, size_t bytes)
+{
+    return p >= base && p - base <= size && size - (p - base) >= bytes;
+}
+
 // Sizes of an instance in each array family.
 struct InstSizes {
     int64_t e, b, c, p, s, m;

@@ -101,3 +101,32 @@ def test_a_single_solve_resumed_anywhere_gives_the_same_bits(capi, precision, n,
         part = run(47 - cut, run(cut))
         for k in whole:
             assert np.array_equal(whole[k], part[k]), (cut, k)
+
+
+def test_device_results_in_any_kind_of_buffer(capi):
+    """Neighbouring ranges of one allocation, NULL, and a misaligned buffer that takes the copies, in one call."""
+    import torch
+    shapes = [(37, 3, 5), (64, 2, 1), (50, 2, 2), (33, 4, 3)]
+    P = [W.random_problem(n, m, q, seed=400 + t) for t, (n, m, q) in enumerate(shapes)]
+    dp = ctypes.POINTER(ctypes.c_double)
+    with capi.Batch(P, W.Params(rho2_over_n=True, precision="mixed", max_iter=20)) as b:
+        b.solve()
+        host = b.wait(want_x=True)
+        size = [n * m * q for n, m, q in shapes]
+        one = torch.full((sum(size) * 8 + 4,), 7, dtype=torch.uint8, device="cuda")
+        res = (capi.admm_result * len(P))()
+        at = [0]
+        for t, r in enumerate(res):
+            off = 8 * at[-1] + (4 if t == 3 else 0)  # the last one misaligned
+            r.x = ctypes.cast(ctypes.c_void_p(one.data_ptr() + off), dp) if t != 1 else None
+            r.on_device = 1
+            at.append(at[-1] + size[t])
+        assert capi._lib.admm_batch_wait(b.h, None, res) in (capi.ADMM_OK, capi.ADMM_ENOTCONVERGED)
+        got = one.cpu().numpy()
+        for t, (n, m, q) in enumerate(shapes):
+            off = 8 * at[t] + (4 if t == 3 else 0)
+            raw = got[off:off + 8 * size[t]]
+            if t == 1:
+                assert np.all(raw == 7)
+            else:
+                assert np.array_equal(raw.copy().view(np.float64).reshape(m, q, n), host[t]["x"])

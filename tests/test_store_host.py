@@ -52,3 +52,10 @@ def test_instance_staging_packs_and_validates(compile_harness):
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stderr
     assert "staging ok" in r.stdout
+
+
+def test_result_buffers_are_held_to_their_allocation(compile_harness):
+    exe = compile_harness("range_holds_check")
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stderr
+    assert "ranges ok" in r.stdout
