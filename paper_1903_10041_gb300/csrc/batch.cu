@@ -202,13 +202,15 @@ void launch_shift_state(const BatchInst *inst, const int *ids, int count, float 
 }
 
 // Shared memory (doubles) of one team: scalar state, double-buffered records
-// of `items` work items, per-warp column maxima, x at k = 0, scratch, and
-// the FP32 zeta + lambda and x1 + nu vectors and the rows' record ranges.
+// of `items` work items, per-warp column maxima, scratch, and in 4-byte words
+// the FP32 zeta + lambda, x1 + nu and x at k = 0 vectors and the rows' record
+// ranges.  No more than the sizes accepted since the first version take: what
+// fits in an SM's shared memory decides which shapes a configuration accepts.
 static size_t team_doubles(int m, int q, int items, int nwt)
 {
     const int mq = m * q;
-    return (size_t)scal_size(m, q) + 2 * (size_t)items * m * 4 + 4 * (size_t)nwt + 24 + mq + kWarpsMax * 8 +
-           2 * ((mq + 1) / 2) + (q + 1) / 2 + 8;
+    return (size_t)scal_size(m, q) + 2 * (size_t)items * m * 4 + 4 * (size_t)nwt + 24 + kWarpsMax * 8 +
+           (3 * mq + q + 1) / 2 + 8;
 }
 
 size_t batch_slice_doubles(int max_m, int max_q)

@@ -129,7 +129,7 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
     const int64_t npairs = (int64_t)q * nv;
     const int items = q + W - 1; // record slots: (row j, warp w) at j + w
 
-    // shared memory: scal | rec[2][items][m][4] | cmax[2][NWT][2] | part[24] | x0s[mq] | scr | uoff | x1nu | rows[q]
+    // shared memory: scal | rec[2][items][m][4] | cmax[2][NWT][2] | part[24] | scr | uoff | x1nu | x0s | rows[q]
     // part: [0], [1] end-of-solve sums; [2] kappa; [3] the adaptation factor of a check; [4] 1/q; [5] n;
     // [16..19] fpar; [20..23] ipar.  Thread 0 keeps these team-wide values current so that the other threads read them
     // instead of each converting and dividing on the FP64 pipe.
@@ -141,11 +141,11 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
     double *part = cmax + 4 * NWT;
     float *fpar = (float *)(part + 16); // rho_1, rho_3, rho_4, the pending mu divisor and 1/q, in FP32
     int *ipar = (int *)(part + 20);     // converged, penalties changed, cold start, log2 of the lanes per pair
-    double *x0s = part + 24;
-    double *scr = x0s + mq;
+    double *scr = part + 24;
     float *uoff = (float *)(scr + kWarpsMax * 8); // [mq] (float)(zeta + lambda)
     float *x1nu = uoff + mq;                      // [mq] (float)(x1 + nu)
-    int *rows = (int *)(x1nu + mq);               // [q] first warp whose range covers row j, how many << 16
+    float *x0s = x1nu + mq;                       // [mq] x at k = 0
+    int *rows = (int *)(x0s + mq);                // [q] first warp whose range covers row j, how many << 16
 
     double *gscal = a.scal + I.off_scal;
     double *out = a.out + (size_t)id * kInfo;
@@ -347,15 +347,15 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
                 const int w = rows[j] & 0xffff; // k = 0 lies in the first warp's piece
                 const double *rb = recs;
                 if constexpr (KIND == TEAM_CLUSTER) rb = cg::this_cluster().map_shared_rank(recs, w / NWT);
-                const double x0 = f32_to_f64_nan(*(const float *)(rb + ((size_t)(j + w) * m + i) * 4 + 3));
-                const double d = x0 - nu[i * q + j];
+                const float x0 = *(const float *)(rb + ((size_t)(j + w) * m + i) * 4 + 3);
+                const double d = f32_to_f64_nan(x0) - nu[i * q + j];
                 x0s[i * q + j] = x0;
                 sum = j == lane ? d : sum + d;
             }
             const double xn = __dmul_rn(warp_sum(sum), part[4]);         // (c), the mean over j; not fused into (h)
             for (int j = lane; j < q; j += 32) {
                 const int pr = i * q + j;
-                const double d = xn - x0s[pr], nun = nu[pr] + d;      // (h)
+                const double d = xn - f32_to_f64_nan(x0s[pr]), nun = nu[pr] + d; // (h)
                 nu[pr] = nun;
                 x1nu[pr] = f64_to_f32_nan(xn + nun);
                 if (check) r4m = max_nonneg(r4m, fabs(d));

@@ -130,3 +130,17 @@ def test_device_results_in_any_kind_of_buffer(capi):
                 assert np.all(raw == 7)
             else:
                 assert np.array_equal(raw.copy().view(np.float64).reshape(m, q, n), host[t]["x"])
+
+
+@pytest.mark.parametrize("n,m,q", [(40, 2, 54), (33, 1, 108)])
+def test_shapes_that_just_fit_a_cta_of_16_warp_teams(capi, n, m, q):
+    """Sixteen one-warp teams side by side need nearly all of an SM's shared memory at these shapes; the bits
+    are those of four in a CTA."""
+    P = [W.random_problem(n, m, q, seed=500 + t) for t in range(20)]
+    x = []
+    for warps in (4, 16):
+        with capi.Batch(P, W.Params(rho2_over_n=True, precision="mixed", max_iter=25)) as b:
+            b.set_config(warps, 0, 1 << 20, 1, 1 << 20)
+            b.solve()
+            x.append([r["x"] for r in b.wait(want_x=True)])
+    assert all(np.array_equal(u, v) for u, v in zip(*x))

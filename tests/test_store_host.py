@@ -59,3 +59,10 @@ def test_result_buffers_are_held_to_their_allocation(compile_harness):
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stderr
     assert "ranges ok" in r.stdout
+
+
+def test_batch_shared_memory_takes_every_shape_it_took(compile_harness):
+    exe = compile_harness("batch_smem_check")
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stderr
+    assert "shared memory ok" in r.stdout
