@@ -128,11 +128,7 @@ SingleShape single_shape(int precision, int m, int q, int64_t rs, int nsm, size_
     // mixed: the wide variant where 256 threads per SM would take more than one
     // pass (see NT at single_kernel).
     sh.wide = (mixed && ncols > (int64_t)nsm * single_threads(precision, 1) * unit) ? 2 : 1;
-    int per_sm = single_blocks_per_sm(precision, m, sh.wide, smem);
-    if (per_sm < 1 && sh.wide == 2) {
-        sh.wide = 1;
-        per_sm = single_blocks_per_sm(precision, m, 1, smem);
-    }
+    const int per_sm = single_blocks_per_sm(precision, m, sh.wide, smem);
     if (per_sm < 1) return sh;
     const int64_t g = std::min<int64_t>((int64_t)nsm * per_sm, std::max<int64_t>(1, ncols / (32 * unit)));
     sh.chunk = ((ncols + g - 1) / g + unit - 1) / unit * unit;
