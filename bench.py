@@ -43,9 +43,10 @@ L2_FLUSH_BYTES = 512 << 20  # > 126 MB L2
 # FP64 peak of GB300 derived from unit counts and clock: 152 SMs x 2 DFMA/clk
 # per SM x 2 flop x 2.07 GHz (the measured DFMA rate is 1.90/clk/SM).
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
-# Conventional FP64 flops of one iteration of the FP64 kernel, counted from
-# its element update (each +, -, *, /, sqrt and cube root counts 1, an FMA 2;
-# comparisons and clamps 0):
+# Conventional FP64 flops of one iteration of the method in FP64, counted with
+# Algorithm 1 as its closed form (each +, -, *, /, sqrt and cube root counts 1, an
+# FMA 2; comparisons and clamps 0).  The kernel does other work for the same
+# result, see fp64_kernel_flops_per_iteration.
 #   every element: the sum over the other sources (m - 1), phi (3), the
 #     lossless parts of C and D (6), its share of the column sums of x and
 #     x - x~ (3);
@@ -72,6 +73,18 @@ def fp64_flops_per_iteration(P) -> int:
             + FLOPS_PER_COLUMN * P.q * P.n)
 
 
+def fp64_kernel_flops_per_iteration(P) -> int:
+    """FP64 flops that the FP64 kernel executes (column64): the root is found in FP32 and refined by two
+    FP64 evaluations of the factored half-derivative, 40 flops (21 instructions) for an element with losses
+    and 14 (7) for one without, and 3 m per column.  Rare closed forms and the per-pair scalar steps are
+    left out."""
+    import numpy as np
+    lossy = int(np.count_nonzero((np.asarray(P.g2) != 0) | (np.asarray(P.g1) != 0)))
+    if getattr(P, "coef_shared", False):
+        lossy *= P.q
+    return 40 * lossy + 14 * (P.elements - lossy) + 3 * P.m * P.q * P.n
+
+
 def workload(cfg: int, precision: str, coef_shared: bool = False):
     from paper_1903_10041_gb300 import workloads as W
     P = W.config(cfg)
@@ -88,14 +101,13 @@ def workload(cfg: int, precision: str, coef_shared: bool = False):
 # figure is reported only while the kernel's sources hash to the build it
 # was taken on (otherwise `traffic` is null).
 NCU_TRAFFIC = {
-    ("phev n=1000 q=50", "fp64"): {"bytes_per_iter": (7196672 + 60160) / 3330, "src": "457c39ff1bdae819"},
-    ("plain n=1e5 m=4 q=20", "mixed"): {"bytes_per_iter": (545884681728 + 173432479744) / 2720, "src": "457c39ff1bdae819"},
+    ("phev n=1000 q=50", "fp64"): {"bytes_per_iter": (7197440 + 55552) / 3330, "src": "88f0c252d3f8e9d8"},
+    ("plain n=1e5 m=4 q=20", "mixed"): {"bytes_per_iter": (545293847808 + 173435627520) / 2720, "src": "88f0c252d3f8e9d8"},
 }
-NCU_TRAFFIC_BATCH = {"bytes_per_element_iter": (1824847392768 + 617704844800) / 76364664590.0, "src": "58ea3e62cb52c56a"}
+NCU_TRAFFIC_BATCH = {"bytes_per_element_iter": (1823401903872 + 617573720576) / 76364664590.0, "src": "91fe1406a0246593"}
 # FP64 pipe utilisation (sm__pipe_fp64_cycles_active, % of peak over the active cycles) of the FP64 solve
-# kernel on the PHEV instance, from an ncu capture of the same build: the counted-flop fraction leaves out
-# the Newton steps of the FP32-seeded roots, conversions, comparisons and the per-pair scalar phase.
-NCU_FP64_PIPE = {("phev n=1000 q=50", "fp64"): {"pct": 59.42, "src": "457c39ff1bdae819"}}
+# kernel on the PHEV instance, from an ncu capture of the same build.
+NCU_FP64_PIPE = {("phev n=1000 q=50", "fp64"): {"pct": 59.37, "src": "88f0c252d3f8e9d8"}}
 
 # Sources each solve kernel is compiled from.
 SINGLE_KERNEL_SOURCES = ("single.cu", "single_cluster.cu", "single_kernel.cuh", "quartic32.cuh", "quartic64.cuh",
@@ -1010,6 +1022,10 @@ def run_single(args, P, par, rank, world, local):
                     "frac": achieved / FP64_PEAK_TFLOPS, "traffic": traffic_per_launch(P, "fp64", iters),
                     "peak_source": "FP64: 152 SMs x 2 DFMA/clk x 2 x 2.07 GHz (derived; measured 1.90 DFMA/clk/SM)",
                     "fp64_pipe_busy": fp64_pipe_busy(P),
+                    # what `achieved` counts is the closed form; of the peak, the kernel's own FP64 flops take
+                    "flops": "Algorithm 1 as its closed form (the kernel finds roots in FP32 and refines them)",
+                    "kernel_fp64_frac": iters * fp64_kernel_flops_per_iteration(P) / per_launch_s / 1e12
+                    / FP64_PEAK_TFLOPS,
                     # algorithmic bytes streamed per second; an instance that fits in L2
                     # (the n=1000 PHEV one) is served mostly from L2, not HBM (see traffic)
                     "streamed_gbs": iters * bytes_per_iteration(P, "fp64") / per_launch_s / 1e9}

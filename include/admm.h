@@ -287,7 +287,8 @@ admm_status admm_solve_noalloc(const admm_problem *prob, const admm_params *para
 typedef struct admm_batch admm_batch;
 typedef struct admm_batch_config {
     int32_t warps_per_cta;        /* 4, 8 or 16 */
-    int32_t ctas_per_sm;          /* 0 = as many as fit */
+    int32_t ctas_per_sm;          /* 0 = as many as fit, which any larger number is cut to (one CTA
+                                     of 8 or 16 warps, two of 4) */
     int64_t small_max_elements;   /* instances with m*q*n <= this go to one-warp teams */
     int32_t cluster_size;         /* 1 (off), 2, 4 or 8: CTAs of a thread-block cluster team */
     int32_t reserved;             /* must be 0 */

@@ -246,8 +246,8 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
             }
             double *rec = recs + (size_t)(j + gw) * m * 4;
             // PLAIN: not a check iteration, not cold, no pending mu divisor (nine iterations in
-            // ten), a normal rho_3, with those branches and their registers compiled out of the loop (not for M = 8,
-            // where two copies spill more than the branches cost)
+            // ten), a normal rho_3, with those branches and their registers compiled out of the
+            // loop (not for M = 8, where two copies spill more than the branches cost)
             auto columns = [&](auto plain) {
                 constexpr bool PLAIN = decltype(plain)::value;
                 const bool chk = !PLAIN && check, cld = !PLAIN && cold;
@@ -339,7 +339,8 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
         // steps (b), (d), (g), (i) per pair, G lanes sharing a pair's records.  Bound by latency (a
         // chain of about 15 FP64 instructions of 64 cycles): comparisons, conversions and the
         // records' row ranges (once per solve) stay off the FP64 pipe and out of the loop.  4096
-        // adaptive solves 767 -> 691 ms, a burst of 48 served solves (n <= 600) 129 -> 104 ms.
+        // adaptive solves 767 -> 691 ms, a burst of 48 served solves (n <= 600) 129 -> 104 ms
+        // (36 bursts spread by 1.6 ms).
         double r2m = 0.0, r3m = 0.0, r4m = 0.0, s1m = 0.0, s2m = 0.0;
         for (int i = NWT - 1 - wl; i < m; i += NWT) {
             double sum = 0.0;
@@ -533,13 +534,18 @@ template <int KIND, int NW, int M, bool ROLL> __device__ void solve_team(const B
     sync_team(); // rank 0 has read every member's shared memory
 }
 
-// Registers: CTAs of 16 warps have 128 a thread; smaller ones take 255, which
-// leaves 8 warps per SM instead of 16 but nothing spilled.  With 8 warps per
-// CTA that is faster at every batch size tried, most where the largest
-// instances' iterations on one CTA are what a batch waits for (150 / 600 / 2000
-// instances x 100 iterations: 38.4 / 58.4 / 66.9 -> 22.4 / 37.7 / 57.1 ms).  12 warps
-// of 168 registers in the place of 16: 4096 adaptive solves 688 -> 673 ms, but a
-// burst of 48 served solves 106 -> 118 ms.
+// Registers: CTAs of 16 warps have 128 a thread and spill (M = 4: 880 bytes
+// stored and 1360 loaded, M = 8: 1660 and 2510); smaller ones take 255, which
+// leaves 8 warps per SM instead of 16 but nothing spilled at M = 4 and 72 / 92 bytes
+// at M = 8.  With 8 warps per CTA that is faster at every batch size tried, most where
+// the largest instances' iterations on one CTA are what a batch waits for (150 /
+// 600 / 2000 instances x 100 iterations: 38.4 / 58.4 / 66.9 -> 22.4 / 37.7 / 57.1 ms).
+// Batches of small instances alone, 8 warps per CTA, CTA teams | one-warp teams, 100
+// iterations, with the whole build before this and the scalar steps above: 4096 of
+// n 50-200, m 2-4, q 1-4 19.0 -> 15.1 | 14.9 -> 9.9 ms; 4096 of n 50-400, m 5-8, q 1-4
+// 49.0 -> 33.9 | 66.9 -> 33.2; 8192 of n 50-150, m 1-2, q 1 16.5 -> 16.0 | 5.1 -> 4.7.
+// 12 warps of 168 registers in the place of 16: 4096 adaptive solves 688 -> 673 ms,
+// but a burst of 48 served solves 106 -> 118 ms.
 template <int NW, int M, bool ROLL>
 __global__ void __launch_bounds__(NW * 32, NW == 16 ? 1 : 8 / NW) batch_kernel(BatchArgs a)
 {

@@ -654,7 +654,7 @@ __device__ __forceinline__ float2 quartic_min32x2(float2 A, float2 B, float2 C, 
 // both branches): both lanes' Cardano root and both lanes' trig roots are found
 // packed, and each lane keeps what its branch needs, instead of one lane after
 // the other through the scalar code (725 -> 284 warp instructions per 64
-// quartics, 2^26 of them 1014 -> 355 us).  The decisions are those of quartic_min32: the branch outside
+// quartics, 2^26 of them 1014 -> 350 us).  The decisions are those of quartic_min32: the branch outside
 // its error bound, the lower minimum where |br| of F(u) - F(v) = (u - v) br
 // exceeds 2e-5 of the sum of its terms' magnitudes (FP32 errs by a few 1e-7
 // of it).  okx, oky: a lane with anything nearer than that, A = 0, or a value that

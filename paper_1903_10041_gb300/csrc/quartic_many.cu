@@ -189,7 +189,7 @@ BadWords g_bad_words;
 // CTAs of the FP32 kernel: a pair per thread up to kPerSm CTAs per SM (eight
 // resident, the rest handed out as others finish), then more pairs per thread,
 // whose next loads run beside the solve.  2^26 quartics: 389 us with a pair per
-// thread and no prefetch, 355 (79 % of HBM) so.
+// thread and no prefetch, 350 (80 % of HBM) so.
 int quartic_grid(int64_t pairs)
 {
     int dev = 0, nsm = 0;

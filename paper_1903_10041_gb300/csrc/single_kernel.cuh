@@ -497,12 +497,13 @@ __device__ __forceinline__ void derive_penalties(const Sm &sm, int n)
 }
 
 // NT: threads of a CTA, one CTA per SM.  FP64 takes 384 (168 registers).  The
-// mixed kernel takes 256 (255 registers, no spills) where one pass covers the
-// columns, and 384 where a thread has several: two CTAs of 256 at 128
-// registers keep a third more warps but spill, and the reloads come back
-// through an L1 that the stage's copies sweep (n = 1e5, m = 4, q = 20: 76.1 ->
-// 66.7 us per iteration; 320 threads 72.3, 448 79.5; n = 10007, m = 6, q = 11:
-// 21.5 -> 18.8).
+// mixed kernel takes 256 (255 registers, at most 32 bytes spilled) where one pass
+// covers the columns, and 384 (168) where a thread has several: two CTAs of 256
+// at 128 registers keep a third more warps but spill about 500 bytes a thread, and
+// the reloads come back through an L1 that the stage's copies sweep (n = 1e5, m = 4,
+// q = 20: 76.1 -> 66.7 us per iteration; 320 threads 72.3, 448 79.5; n = 10007, m =
+// 6, q = 11: 21.5 -> 18.8).  384 spill 156 bytes stored and 88 loaded at M = 4, 360 and
+// 392 at M = 8, none at M = 2.
 template <int M, int PREC, int NT, bool CL>
 __global__ void __launch_bounds__(NT, 1) single_kernel(SingleArgs a)
 {
@@ -616,9 +617,9 @@ __global__ void __launch_bounds__(NT, 1) single_kernel(SingleArgs a)
                 const int kn = min(ke, n); // padding columns k >= n are skipped
                 const bool tiny_c = tiny_rho3(rho3);
                 // PLAIN: not a check iteration, not cold, no pending mu divisor (nine iterations in
-                // ten), a normal rho_3, with those branches and their registers compiled out of the loop (n = 1e5,
-                // m = 4, q = 20: 91.3 -> 80.2 us per iteration).  Not for M = 8, where two copies
-                // spill more than the branches cost (m = 6: 23.0 -> 25.9).
+                // ten), a normal rho_3, with those branches and their registers compiled out of the
+                // loop (n = 1e5, m = 4, q = 20: 91.3 -> 80.2 us per iteration).  Not for M = 8, where
+                // two copies spill more than the branches cost (m = 6: 23.0 -> 25.9).
                 auto columns = [&](auto plain) {
                     constexpr bool PLAIN = decltype(plain)::value;
                     const bool chk = !PLAIN && check, cld = !PLAIN && cold;
