@@ -301,7 +301,7 @@ __global__ void batch_export_kernel(const BatchInst *inst, const BatchExport *ex
         for (int i = threadIdx.x; i < I.m; i += blockDim.x) e.x1[i] = scal[I.off_scal + 5 * mq + i];
 }
 
-// Allocation that holds device pointer p, by the driver (loaded by the runtime already).
+// Allocation that holds device pointer p, asked of the CUDA driver API (loaded by the runtime already).
 bool allocation_of(const void *p, uintptr_t &base, size_t &size)
 {
     using Fn = CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr);
